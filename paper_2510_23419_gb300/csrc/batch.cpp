@@ -79,9 +79,11 @@ double est_cost(const pb_instance* I, int R, int S, int form, double* compute = 
     const double upd = (double)I->N * R * std::max(1, S);
     double c, lat = 0.0;
     if (I->topo == PB_TOPO_EA3D) {
-        // resident form: the fast tiles (L = 8, 16, 32) vs the generic tile, +-1 vs FP32
+        // resident form: +-1 by the sites per spin word; FP32 the fast tiles (L = 8, 16, 32) or the generic one
         const bool fast = I->L == 8 || I->L == 16 || I->L == 32, f32 = I->jtype == PB_J_F32;
-        const double rate = form == PB_FORM_PLAIN ? 9e10 : fast ? (f32 ? 6e11 : 8.5e11) : (f32 ? 4e11 : 6e11);
+        const double rate = form == PB_FORM_PLAIN ? 9e10
+                            : f32                 ? (fast ? 6e11 : 4e11)
+                                                  : (I->L % 8 == 0 ? 1.2e12 : 9e11);
         c = upd / rate;
     } else if (I->topo == PB_TOPO_CSR) {
         c = upd * std::max(1, I->maxdeg) / 4e11;

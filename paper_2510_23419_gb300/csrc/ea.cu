@@ -11,6 +11,7 @@
 //    neighbour word is read from shared memory.
 //  * plain: spins in global memory, one launch per colour class and sweep,
 //    plus one energy/best launch per sweep.
+#include "ea_bits.cuh"
 #include "ea_fast.cuh"
 #include "ea_kernels.cuh"
 #include <mutex>
@@ -32,12 +33,11 @@ struct TileCtx {
     uint32_t tq;                 // Philox counter word 2 = replica quad index
 };
 
-template <int LT, int WTT>
 __device__ __forceinline__ TileCtx tile_ctx(const EaJob& job, int tile)
 {
     TileCtx g;
-    g.L = LT ? LT : job.inst.L;
-    g.WT = WTT ? WTT : job.WT;
+    g.L = job.inst.L;
+    g.WT = job.WT;
     g.h2 = g.L >> 1;
     g.half = g.h2 * g.L * g.L;
     g.N = 2 * g.half;
@@ -64,8 +64,7 @@ __device__ __forceinline__ TileCtx tile_ctx(const EaJob& job, int tile)
 
 // Sum 4 per-thread values over the lanes that hold the same w, then store the
 // warp's sums in part[warp][4w + b].
-template <typename T>
-__device__ __forceinline__ void warp_partials(const TileCtx& g, T v0, T v1, T v2, T v3, T* part)
+__device__ __forceinline__ void warp_partials(const TileCtx& g, float v0, float v1, float v2, float v3, float* part)
 {
     for (int o = g.WT; o < 32; o <<= 1) {
         v0 += __shfl_xor_sync(0xFFFFFFFFu, v0, o);
@@ -74,39 +73,19 @@ __device__ __forceinline__ void warp_partials(const TileCtx& g, T v0, T v1, T v2
         v3 += __shfl_xor_sync(0xFFFFFFFFu, v3, o);
     }
     if (g.lane < g.WT) {
-        T* p = part + g.warp * 4 * g.WT + 4 * g.lane;
+        float* p = part + g.warp * 4 * g.WT + 4 * g.lane;
         p[0] = v0; p[1] = v1; p[2] = v2; p[3] = v3;
-    }
-}
-
-// Byte-lane counts (<= 255 each) -> four int32 partials.
-__device__ __forceinline__ void warp_partials_bytes(const TileCtx& g, uint32_t acc, int32_t* part)
-{
-    uint32_t a = acc & 0x00FF00FFu;         // replicas 0 and 2 in 16-bit lanes
-    uint32_t b = (acc >> 8) & 0x00FF00FFu;  // replicas 1 and 3
-    for (int o = g.WT; o < 32; o <<= 1) {
-        a += __shfl_xor_sync(0xFFFFFFFFu, a, o);
-        b += __shfl_xor_sync(0xFFFFFFFFu, b, o);
-    }
-    if (g.lane < g.WT) {
-        int32_t* p = part + g.warp * 4 * g.WT + 4 * g.lane;
-        p[0] = (int32_t)(a & 0xFFFFu);
-        p[1] = (int32_t)(b & 0xFFFFu);
-        p[2] = (int32_t)(a >> 16);
-        p[3] = (int32_t)(b >> 16);
     }
 }
 
 // Merge the thread's words of both colours into a global state buffer for the
 // replicas that `flags` selects (byte b = 1: replica 4w + b of each word;
 // 0x01010101: all), with the same word partition as the half-sweeps.
-template <int LT, int WTT>
 __device__ __forceinline__ void tile_store_words(const TileCtx& g, const uint32_t* sp, uint32_t* gdst, int tile,
                                                  uint32_t flags)
 {
     if (!g.active || flags == 0u) return;
-    const int L = LT ? LT : g.L;
-    const int WT = WTT ? WTT : g.WT;
+    const int L = g.L, WT = g.WT;
     const int h2 = L >> 1;
     const int half = h2 * L * L;
 #pragma unroll 1
@@ -123,51 +102,25 @@ __device__ __forceinline__ void tile_store_words(const TileCtx& g, const uint32_
     }
 }
 
-template <int LT, int WTT, int JT, bool HH>
+// Generic tile of real couplings: any even L <= 32 without a compile-time tile.
 __device__ void ea_tile(const EaJob& job, int tile, unsigned char* smem)
 {
-    const TileCtx g = tile_ctx<LT, WTT>(job, tile);
-    const int L = LT ? LT : g.L;
-    const int WT = WTT ? WTT : g.WT;
+    const TileCtx g = tile_ctx(job, tile);
+    const int L = g.L, WT = g.WT;
     const int h2 = L >> 1;
     const int half = h2 * L * L;
     const int N = 2 * half;
     const int nrep = 4 * WT;
 
     // ---- shared memory carve-up (must match ea_resident_smem) ----
-    unsigned char* p = smem;
-    uint32_t* sp = reinterpret_cast<uint32_t*>(p);
-    p += (size_t)N * WT * 4;
-    uint8_t* sjb = nullptr;
-    int8_t* sh8 = nullptr;
-    if (JT == PB_J_PM1_I8) {
-        sjb = p;
-        p += (N + 15) / 16 * 16;
-        if (HH) {
-            sh8 = reinterpret_cast<int8_t*>(p);
-            p += (N + 15) / 16 * 16;
-        }
-    }
-    const int tabw = (JT == PB_J_PM1_I8) ? (HH ? job.nF : 64) : 0;
-    const int tabw4 = (tabw + 3) / 4 * 4;
-    uint32_t* stab = reinterpret_cast<uint32_t*>(p);
-    p += (size_t)2 * tabw4 * 4;
-    int32_t* spart_i = reinterpret_cast<int32_t*>(p);
-    float* spart_f = reinterpret_cast<float*>(p);
-    p += (size_t)kResidentWarps * nrep * 4;
-    int32_t* spart_h = reinterpret_cast<int32_t*>(p);
-    if (JT == PB_J_PM1_I8 && HH) p += (size_t)kResidentWarps * nrep * 4;
-    uint8_t* sflag = p;
+    uint32_t* sp = reinterpret_cast<uint32_t*>(smem);
+    float* spart = reinterpret_cast<float*>(sp + (size_t)N * WT);
+    uint8_t* sflag = reinterpret_cast<uint8_t*>(spart + kResidentWarps * nrep);
 
     const uint32_t key0 = job.key0, key1 = job.key1;
     const int t = g.t;
 
-    // ---- instance data and initial state (tag 1) ----
-    if (JT == PB_J_PM1_I8) {
-        for (int i = t; i < N; i += kResidentThreads) sjb[i] = job.inst.jbits[i];
-        if (HH)
-            for (int i = t; i < N; i += kResidentThreads) sh8[i] = job.inst.h8[i];
-    }
+    // ---- initial state (tag 1) ----
     for (int j = t; j < N * WT; j += kResidentThreads) {
         if (job.resume) {  // resumed run: the given state, in the tile layout of final_words
             sp[j] = job.final_words[(size_t)tile * N * WT + j];
@@ -178,37 +131,18 @@ __device__ void ea_tile(const EaJob& job, int tile, unsigned char* smem)
         const int c = ck >= half ? 1 : 0;
         const int k = ck - c * half;
         const U4 r = philox10((uint32_t)k, 0u, (uint32_t)(tile * WT + w2), (kTagInit << 24) | (uint32_t)c, key0, key1);
-        sp[j] = (JT == PB_J_PM1_I8) ? ((r.x >> 31) | ((r.y >> 31) << 8) | ((r.z >> 31) << 16) | ((r.w >> 31) << 24))
-                                    : f32_word(r.x >> 31, r.y >> 31, r.z >> 31, r.w >> 31);
+        sp[j] = f32_word(r.x >> 31, r.y >> 31, r.z >> 31, r.w >> 31);
     }
 
-    auto build_table = [&](int s, int buf) {
-        if (JT != PB_J_PM1_I8) return;
-        const int level = s / job.step;
-        const uint32_t* row = job.table + (size_t)level * job.nF;
-        if (!HH) {
-            if (t < 64) {
-                const int F = 6 - 2 * __popc((unsigned)t);
-                stab[buf * tabw4 + t] = row[F - job.fmin];
-            }
-        } else {
-            for (int f = t; f < job.nF; f += kResidentThreads) stab[buf * tabw4 + f] = row[f];
-        }
-    };
-
     // One colour class: update (decide = true) or only accumulate the energy
-    // terms (decide = false, for the initial state).  Returns the thread's
-    // per-replica accumulators: PM1 -> unsatisfied-bond counts in byte lanes
-    // (class 1 only) and h.m sums; F32 -> -m F (class 1) and -h m (class 0).
-    auto half_sweep = [&](int c, int s, bool decide, uint32_t& uacc, int32_t (&hm)[4], float (&ef)[4]) {
+    // terms (decide = false, for the initial state): -m F (class 1) and -h m
+    // (class 0) per replica.
+    auto half_sweep = [&](int c, int s, bool decide, float (&ef)[4]) {
         if (!g.active) return;
         const uint32_t* o = sp + (size_t)(1 - c) * half * WT;
         uint32_t* own = sp + (size_t)c * half * WT;
         const uint32_t c3 = (kTagDecision << 24) | (uint32_t)c;
-        const int buf = s & 1;
-        const uint32_t* tab = stab + buf * tabw4;
-        float cexp = 0.0f;
-        if (JT == PB_J_F32) cexp = f32_cexp(job.betaf[s / job.step]);
+        const float cexp = f32_cexp(job.betaf[s / job.step]);
         for (int zp = 0; zp < (g.zstep == 1 ? 2 : 1); ++zp) {
             const int z0 = (g.zstep == 1) ? zp : g.zfirst;
             const int px = (c + g.y + z0) & 1;
@@ -221,174 +155,94 @@ __device__ void ea_tile(const EaJob& job, int tile, unsigned char* smem)
                 const int kw = k * WT + g.w;
                 const int ozp = (z + 1 == L) ? -(L - 1) * sz : sz;
                 const int ozm = (z == 0) ? (L - 1) * sz : -sz;
-                const uint32_t n0 = o[kw + oxp], n1 = o[kw + oxm], n2 = o[kw + oyp];
-                const uint32_t n3 = o[kw + oym], n4 = o[kw + ozp], n5 = o[kw + ozm];
-                if (JT == PB_J_PM1_I8) {
-                    const uint32_t X = ea_pattern(n0, n1, n2, n3, n4, n5, sjb[c * half + k]);
-                    uint32_t snew;
-                    if (decide) {
-                        const U4 r = philox10((uint32_t)k, (uint32_t)s, g.tq, c3, key0, key1);
-                        if (!HH) {
-                            const unsigned char* tb = reinterpret_cast<const unsigned char*>(tab);
-                            const uint32_t T0 = *reinterpret_cast<const uint32_t*>(tb + (X & 0xFFu));
-                            const uint32_t T1 = *reinterpret_cast<const uint32_t*>(tb + ((X >> 8) & 0xFFu));
-                            const uint32_t T2 = *reinterpret_cast<const uint32_t*>(tb + ((X >> 16) & 0xFFu));
-                            const uint32_t T3 = *reinterpret_cast<const uint32_t*>(tb + (X >> 24));
-                            snew = decide_bit(r.x, T0) | (decide_bit(r.y, T1) << 8) | (decide_bit(r.z, T2) << 16) |
-                                   (decide_bit(r.w, T3) << 24);
-                        } else {
-                            const int hi = sh8[c * half + k];
-                            const int base = 6 + hi - job.fmin;  // index of F = 6 - 2n + h
-                            const uint32_t T0 = tab[base - 2 * __popc(X & 0xFCu)];
-                            const uint32_t T1 = tab[base - 2 * __popc((X >> 8) & 0xFCu)];
-                            const uint32_t T2 = tab[base - 2 * __popc((X >> 16) & 0xFCu)];
-                            const uint32_t T3 = tab[base - 2 * __popc((X >> 24) & 0xFCu)];
-                            snew = decide_bit(r.x, T0) | (decide_bit(r.y, T1) << 8) | (decide_bit(r.z, T2) << 16) |
-                                   (decide_bit(r.w, T3) << 24);
-                        }
-                        own[kw] = snew;
-                    } else {
-                        snew = own[kw];
-                    }
-                    if (c == 1) uacc += ea_popc6_bytes(X ^ (snew * 0xFCu));
-                    if (HH) {
-                        const int hi = sh8[c * half + k];
-                        hm[0] += (snew & 0x1u) ? -hi : hi;
-                        hm[1] += (snew & 0x100u) ? -hi : hi;
-                        hm[2] += (snew & 0x10000u) ? -hi : hi;
-                        hm[3] += (snew & 0x1000000u) ? -hi : hi;
-                    }
+                const uint32_t nb[6] = {o[kw + oxp], o[kw + oxm], o[kw + oyp], o[kw + oym], o[kw + ozp], o[kw + ozm]};
+                const size_t site = (size_t)c * half + k;
+                const float4 ja = __ldg(reinterpret_cast<const float4*>(job.inst.j6) + 2 * site);
+                const float4 jb = __ldg(reinterpret_cast<const float4*>(job.inst.j6) + 2 * site + 1);
+                const float jv[6] = {ja.x, ja.y, ja.z, ja.w, jb.x, jb.y};
+                const float hv = jb.z;  // the site's field rides in the coupling vector
+                uint32_t snew = 0;
+                float F[4];
+#pragma unroll
+                for (int b = 0; b < 4; ++b) F[b] = ea_field_f32(jv, hv, nb, b);
+                if (decide) {
+                    const U4 r = philox10((uint32_t)k, (uint32_t)s, g.tq, c3, key0, key1);
+                    snew = decide_f32_word(r.x, r.y, r.z, r.w, F[0], F[1], F[2], F[3], cexp);
+                    own[kw] = snew;
                 } else {
-                    const size_t site = (size_t)c * half + k;
-                    const float4 ja = __ldg(reinterpret_cast<const float4*>(job.inst.j6) + 2 * site);
-                    const float4 jb = __ldg(reinterpret_cast<const float4*>(job.inst.j6) + 2 * site + 1);
-                    const float jv[6] = {ja.x, ja.y, ja.z, ja.w, jb.x, jb.y};
-                    const float hv = jb.z;  // the site's field rides in the coupling vector
-                    const uint32_t nb[6] = {n0, n1, n2, n3, n4, n5};
-                    uint32_t snew = 0;
-                    float F[4];
+                    snew = own[kw];
+                }
 #pragma unroll
-                    for (int b = 0; b < 4; ++b) F[b] = ea_field_f32(jv, hv, nb, b);
-                    if (decide) {
-                        const U4 r = philox10((uint32_t)k, (uint32_t)s, g.tq, c3, key0, key1);
-                        snew = decide_f32_word(r.x, r.y, r.z, r.w, F[0], F[1], F[2], F[3], cexp);
-                        own[kw] = snew;
-                    } else {
-                        snew = own[kw];
-                    }
-#pragma unroll
-                    for (int b = 0; b < 4; ++b) {
-                        const bool dn = f32_minus(snew, b);  // m = -1
-                        if (c == 1)
-                            ef[b] += dn ? F[b] : -F[b];           // -m F
-                        else if (job.inst.has_h)
-                            ef[b] += dn ? hv : -hv;               // -h m
-                    }
+                for (int b = 0; b < 4; ++b) {
+                    const bool dn = f32_minus(snew, b);  // m = -1
+                    if (c == 1)
+                        ef[b] += dn ? F[b] : -F[b];           // -m F
+                    else if (job.inst.has_h)
+                        ef[b] += dn ? hv : -hv;               // -h m
                 }
             }
         }
     };
 
-    // Collect the per-replica energy of the state now in shared memory.
-    auto energy_partials = [&](uint32_t uacc, const int32_t (&hm)[4], const float (&ef)[4]) {
-        if (JT == PB_J_PM1_I8) {
-            warp_partials_bytes(g, uacc, spart_i);
-            if (HH) warp_partials<int32_t>(g, hm[0], hm[1], hm[2], hm[3], spart_h);
-        } else {
-            warp_partials<float>(g, ef[0], ef[1], ef[2], ef[3], spart_f);
-        }
-    };
     // Thread r < nrep: energy of replica r from the warp partials (fixed order).
-    auto energy_of = [&](int r, int32_t& Ei, float& Ef) {
-        if (JT == PB_J_PM1_I8) {
-            int32_t U = 0, H = 0;
-            for (int v = 0; v < kResidentWarps; ++v) {
-                U += spart_i[v * nrep + r];
-                if (HH) H += spart_h[v * nrep + r];
-            }
-            // E = -(#satisfied - #unsatisfied) - sum h m = -(3N - 2U) - sum h m
-            Ei = -(3 * N - 2 * U) - H;
-        } else {
-            float E = 0.0f;
-            for (int v = 0; v < kResidentWarps; ++v) E += spart_f[v * nrep + r];
-            Ef = E;
-        }
+    auto energy_of = [&](int r) {
+        float E = 0.0f;
+        for (int v = 0; v < kResidentWarps; ++v) E += spart[v * nrep + r];
+        return E;
     };
 
     // ---- initial energy; the initial state is the first best state (unless resumed) ----
-    const int s_first = job.s0 < job.S ? job.s0 : 0;
-    build_table(s_first, s_first & 1);
     __syncthreads();
     {
-        uint32_t uacc = 0;
-        int32_t hm[4] = {0, 0, 0, 0};
         float ef[4] = {0.f, 0.f, 0.f, 0.f};
-        half_sweep(0, 0, false, uacc, hm, ef);
-        half_sweep(1, 0, false, uacc, hm, ef);
-        energy_partials(uacc, hm, ef);
+        half_sweep(0, 0, false, ef);
+        half_sweep(1, 0, false, ef);
+        warp_partials(g, ef[0], ef[1], ef[2], ef[3], spart);
     }
     __syncthreads();
-    int32_t bestEi = 0, hit = -1, bsweep = -1;
-    float bestEf = 0.0f;
-    if (t < nrep) energy_of(t, bestEi, bestEf);
+    int32_t hit = -1, bsweep = -1;
+    float bestE = 0.0f;
+    if (t < nrep) bestE = energy_of(t);
     if (job.resume) {  // the running best carried over
         if (t < nrep) {
             const int r = tile * nrep + t;
-            if (JT == PB_J_PM1_I8)
-                bestEi = job.E_best_i[r];
-            else
-                bestEf = job.E_best_f[r];
+            bestE = job.E_best_f[r];
             bsweep = job.best_sweep[r];
         }
     } else {
-        tile_store_words<LT, WTT>(g, sp, job.best_words, tile, 0x01010101u);
+        tile_store_words(g, sp, job.best_words, tile, 0x01010101u);
     }
 
     // ---- sweeps ----
     const bool stop_mode = job.has_target == 2;
     for (int s = job.s0; s < job.S; ++s) {
-        uint32_t uacc = 0;
-        int32_t hm[4] = {0, 0, 0, 0};
         float ef[4] = {0.f, 0.f, 0.f, 0.f};
-        half_sweep(0, s, true, uacc, hm, ef);
+        half_sweep(0, s, true, ef);
         __syncthreads();
-        half_sweep(1, s, true, uacc, hm, ef);
-        energy_partials(uacc, hm, ef);
-        if (s + 1 < job.S) build_table(s + 1, (s + 1) & 1);
+        half_sweep(1, s, true, ef);
+        warp_partials(g, ef[0], ef[1], ef[2], ef[3], spart);
         __syncthreads();
         if (t < nrep) {
-            int32_t Ei = 0;
-            float Ef = 0.0f;
-            energy_of(t, Ei, Ef);
+            const float E = energy_of(t);
             const bool live = job.has_target != 2 || hit < 0;  // stop mode: the best is frozen at the target
-            bool imp;
-            if (JT == PB_J_PM1_I8) {
-                imp = live && Ei < bestEi;
-                if (imp) bestEi = Ei;
-                if (job.has_target && hit < 0 && Ei <= job.target_i) hit = s;
-            } else {
-                imp = live && Ef < bestEf;
-                if (imp) bestEf = Ef;
-                if (job.has_target && hit < 0 && Ef <= job.target_f) hit = s;
-            }
+            const bool imp = live && E < bestE;
+            if (imp) bestE = E;
+            if (job.has_target && hit < 0 && E <= job.target_f) hit = s;
             if (imp) bsweep = s;
             sflag[t] = imp ? 1 : 0;
         }
         __syncthreads();
         const uint32_t f = reinterpret_cast<const uint32_t*>(sflag)[g.w];
-        tile_store_words<LT, WTT>(g, sp, job.best_words, tile, f);
+        tile_store_words(g, sp, job.best_words, tile, f);
         // stop mode: the tile ends once all its replicas (padding included) have reached the target
         if (stop_mode && __syncthreads_and(t >= nrep || hit >= 0 || tile * nrep + t >= job.R)) break;
     }
 
     // ---- results ----
-    tile_store_words<LT, WTT>(g, sp, job.final_words, tile, 0x01010101u);
+    tile_store_words(g, sp, job.final_words, tile, 0x01010101u);
     if (t < nrep) {
         const int r = tile * nrep + t;
-        if (JT == PB_J_PM1_I8)
-            job.E_best_i[r] = bestEi;
-        else
-            job.E_best_f[r] = bestEf;
+        job.E_best_f[r] = bestE;
         job.best_sweep[r] = bsweep;
         job.hit_sweep[r] = hit;
     }
@@ -404,7 +258,7 @@ __device__ void ea_tile(const EaJob& job, int tile, unsigned char* smem)
 // of the same batch) start at once, so that kernel's CTAs take the SMs this
 // one leaves as its list runs out.
 template <int K>
-__global__ void __launch_bounds__(kResidentThreads, 1)
+__global__ void __launch_bounds__(K <= kEaKernelPm1Split ? kBitsThreads : kResidentThreads, 1)
     ea_resident_kernel(const EaJob* __restrict__ jobs, const EaWork* __restrict__ work, int n_work, int* counter)
 {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -418,34 +272,50 @@ __global__ void __launch_bounds__(kResidentThreads, 1)
         if (item >= n_work) break;
         const EaWork wk = work[item];
         const EaJob& job = jobs[wk.job];
-        if constexpr (K == kEaKernelPm1) {
-            if (wk.path == kEaPathFieldsGeneric)
-                ea_tile<0, 0, PB_J_PM1_I8, true>(job, wk.tile, smem);
-            else if (wk.path == kEaPathFast32)
-                ea_tile_fast<32, 1, PB_J_PM1_I8>(job, wk.tile, smem);
-            else if (wk.path == kEaPathFast16)
-                ea_tile_fast<16, 4, PB_J_PM1_I8>(job, wk.tile, smem);
-            else if (wk.path == kEaPathFast8)
-                ea_tile_fast<8, 16, PB_J_PM1_I8>(job, wk.tile, smem);
-            else if (wk.path == kEaPathFast24)
-                ea_tile_fast<24, 1, PB_J_PM1_I8>(job, wk.tile, smem);
-            else if (wk.path == kEaPathGen12)
-                ea_tile<12, 4, PB_J_PM1_I8, false>(job, wk.tile, smem);
-            else
-                ea_tile<0, 0, PB_J_PM1_I8, false>(job, wk.tile, smem);
+        if constexpr (K == kEaKernelPm1 || K == kEaKernelPm1Split) {
+            __shared__ __align__(256) unsigned char s_tab[768];  // threshold rows (EaBitTile::put_entry)
+#define PB_BITS(G, CPT, COL, HH)                                  \
+    case ea_bits_path(G, CPT, COL, HH):                           \
+        ea_tile_bits<G, CPT, COL, HH>(job, wk.tile, smem, s_tab); \
+        break
+            if constexpr (K == kEaKernelPm1) {
+                switch (wk.path) {
+                    PB_BITS(8, 8, true, false);
+                    PB_BITS(8, 8, false, false);
+                    PB_BITS(4, 4, true, false);
+                    PB_BITS(4, 4, false, false);
+                    PB_BITS(2, 2, true, false);
+                    PB_BITS(2, 2, false, false);
+                    PB_BITS(8, 8, false, true);
+                    PB_BITS(4, 4, false, true);
+                    PB_BITS(2, 2, false, true);
+                }
+            } else {
+                switch (wk.path) {
+                    PB_BITS(8, 4, true, false);
+                    PB_BITS(8, 2, true, false);
+                    PB_BITS(8, 1, true, false);
+                    PB_BITS(4, 2, true, false);
+                    PB_BITS(4, 1, true, false);
+                    PB_BITS(2, 1, true, false);
+                    PB_BITS(8, 1, true, true);
+                    PB_BITS(4, 1, true, true);
+                    PB_BITS(2, 1, true, true);
+                }
+            }
+#undef PB_BITS
         } else {
-            // the compile-time L = 12 shape in either FP32 kernel makes it spill: its tiles
-            // run the generic tile, as do L = 24 tiles in the first kernel
+            // L = 24 tiles in the first kernel run the generic tile
             if (K == kEaKernelF32 && wk.path == kEaPathFast32)
-                ea_tile_fast<32, 1, PB_J_F32>(job, wk.tile, smem);
+                ea_tile_fast<32, 1>(job, wk.tile, smem);
             else if (K == kEaKernelF32L24 && wk.path == kEaPathFast24)
-                ea_tile_fast<24, 1, PB_J_F32>(job, wk.tile, smem);
+                ea_tile_fast<24, 1>(job, wk.tile, smem);
             else if (wk.path == kEaPathFast16)
-                ea_tile_fast<16, 4, PB_J_F32>(job, wk.tile, smem);
+                ea_tile_fast<16, 4>(job, wk.tile, smem);
             else if (wk.path == kEaPathFast8)
-                ea_tile_fast<8, 16, PB_J_F32>(job, wk.tile, smem);
+                ea_tile_fast<8, 16>(job, wk.tile, smem);
             else
-                ea_tile<0, 0, PB_J_F32, false>(job, wk.tile, smem);
+                ea_tile(job, wk.tile, smem);
         }
     }
 }
@@ -747,6 +617,42 @@ __global__ void __launch_bounds__(256) ea_readout_kernel(EaJob job, const uint32
     out[j] = minus ? (int8_t)-1 : (int8_t)1;
 }
 
+// The same for one bit per spin (job.groups): a thread writes 2 V consecutive sites
+// of one replica, i.e. V words of both classes give a bit each.  Reads and writes are
+// whole words and whole rows; a byte per thread from the byte layout took 0.4 ms per
+// state set at L = 32 and 1024 replicas.
+template <int V>
+__global__ void __launch_bounds__(256) ea_readout_bits_kernel(EaJob job, const uint32_t* __restrict__ words,
+                                                              int8_t* __restrict__ out, int blocks_per_replica)
+{
+    const int L = job.inst.L, h2 = L >> 1, hv = h2 / V, WT = job.WT;
+    const int r = blockIdx.x / blocks_per_replica;
+    const int j = (blockIdx.x - r * blocks_per_replica) * 256 + threadIdx.x;
+    if (j >= hv * L * L) return;
+    const int row = j / hv, q0 = (j - row * hv) * V;
+    const int z = row / L, y = row - z * L;
+    const int Z = L / job.groups, nw = h2 * L * Z;
+    const int g = z / Z, wi = q0 + h2 * (y + L * (z - g * Z));
+    const int quad = r >> 2, tile = quad / WT, w = quad - tile * WT;
+    const int sh = 8 * (r & 3) + g;
+    const int even = (y + z) & 1;  // the class whose sites of this row have an even x
+    const uint32_t* p0 = words + (((size_t)tile * 2 + even) * nw + wi) * WT + w;
+    const uint32_t* p1 = words + (((size_t)tile * 2 + 1 - even) * nw + wi) * WT + w;
+    uint16_t v[V];
+#pragma unroll
+    for (int k = 0; k < V; ++k) {
+        const uint32_t a = (p0[k * WT] >> sh) & 1u, b = (p1[k * WT] >> sh) & 1u;
+        v[k] = (uint16_t)(0x0101u + a * 0x00FEu + b * 0xFE00u);  // 0x01 = +1, 0xFF = -1
+    }
+    int8_t* dst = out + (size_t)r * job.inst.N + (size_t)row * L + 2 * q0;
+    if constexpr (V == 4)
+        *reinterpret_cast<uint2*>(dst) = make_uint2(v[0] | ((uint32_t)v[1] << 16), v[2] | ((uint32_t)v[3] << 16));
+    else if constexpr (V == 2)
+        *reinterpret_cast<uint32_t*>(dst) = v[0] | ((uint32_t)v[1] << 16);
+    else
+        *reinterpret_cast<uint16_t*>(dst) = v[0];
+}
+
 // E = -sum_{d,i} J[d][i] m_i m_{i+d} - sum_i h_i m_i, one block per replica;
 // int64 for PM1, FP64 for F32 (the only FP64 on the device).
 template <int JT>
@@ -871,20 +777,21 @@ cudaError_t ea_resident_set_smem(int kernel, size_t smem)
     std::lock_guard<std::mutex> lock(mu);
     size_t* cur = (dev >= 0 && dev < 64) ? &current[kernel][dev] : nullptr;
     if (cur && smem <= *cur) return cudaSuccess;
-    const cudaError_t e = kernel == kEaKernelPm1   ? ea_resident_attr<kEaKernelPm1>(smem)
-                          : kernel == kEaKernelF32 ? ea_resident_attr<kEaKernelF32>(smem)
-                                                   : ea_resident_attr<kEaKernelF32L24>(smem);
+    const cudaError_t e = kernel == kEaKernelPm1        ? ea_resident_attr<kEaKernelPm1>(smem)
+                          : kernel == kEaKernelPm1Split ? ea_resident_attr<kEaKernelPm1Split>(smem)
+                          : kernel == kEaKernelF32      ? ea_resident_attr<kEaKernelF32>(smem)
+                                                        : ea_resident_attr<kEaKernelF32L24>(smem);
     if (e == cudaSuccess && cur) *cur = smem;
     return e;
 }
 
 cudaError_t ea_launch_resident(int kernel, const EaJob* d_jobs, const EaWork* d_work, int n_work, int* d_counter,
-                               size_t smem, int grid, bool after_previous, cudaStream_t st)
+                               size_t smem, int grid, int threads, bool after_previous, cudaStream_t st)
 {
     if (kernel < 0 || kernel >= kEaKernels) return cudaErrorInvalidValue;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3(kResidentThreads);
+    cfg.blockDim = dim3((unsigned)threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
@@ -896,6 +803,8 @@ cudaError_t ea_launch_resident(int kernel, const EaJob* d_jobs, const EaWork* d_
     }
     if (kernel == kEaKernelPm1)
         return cudaLaunchKernelEx(&cfg, ea_resident_kernel<kEaKernelPm1>, d_jobs, d_work, n_work, d_counter);
+    if (kernel == kEaKernelPm1Split)
+        return cudaLaunchKernelEx(&cfg, ea_resident_kernel<kEaKernelPm1Split>, d_jobs, d_work, n_work, d_counter);
     if (kernel == kEaKernelF32)
         return cudaLaunchKernelEx(&cfg, ea_resident_kernel<kEaKernelF32>, d_jobs, d_work, n_work, d_counter);
     return cudaLaunchKernelEx(&cfg, ea_resident_kernel<kEaKernelF32L24>, d_jobs, d_work, n_work, d_counter);
@@ -948,6 +857,18 @@ cudaError_t ea_launch_plain_energy(const EaJob& job, int s, bool init, cudaStrea
 
 cudaError_t ea_launch_readout(const EaJob& job, const uint32_t* words, int8_t* out_pm, double* out_E, cudaStream_t st)
 {
+    if (job.groups) {
+        const int h2 = job.inst.L / 2, V = h2 % 4 == 0 ? 4 : (h2 % 2 == 0 ? 2 : 1);
+        const int bpr = (h2 / V * job.inst.L * job.inst.L + 255) / 256;
+        const unsigned grid = (unsigned)bpr * (unsigned)job.R;
+        if (V == 4)
+            ea_readout_bits_kernel<4><<<grid, 256, 0, st>>>(job, words, out_pm, bpr);
+        else if (V == 2)
+            ea_readout_bits_kernel<2><<<grid, 256, 0, st>>>(job, words, out_pm, bpr);
+        else
+            ea_readout_bits_kernel<1><<<grid, 256, 0, st>>>(job, words, out_pm, bpr);
+        return cudaGetLastError();
+    }
     const long long n = (long long)job.R * job.inst.N;
     ea_readout_kernel<<<blocks_for(n, 256), 256, 0, st>>>(job, words, out_pm);
     if (job.inst.jtype == PB_J_PM1_I8)

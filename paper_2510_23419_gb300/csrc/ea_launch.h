@@ -35,67 +35,158 @@ struct EaJob {
     int32_t s0;               // first sweep (resident form: > 0 only for a resumed run)
     int32_t resume;           // resident form: the initial state is final_words, the running best
                               // (best_words, E_best_*, best_sweep) is given
+    int32_t groups;           // 0: state buffers in the byte layout above; else (resident +-1 runs) one bit
+                              // per spin, `groups` sites per word: word ((tile*2 + c)*nw + wi)*WT + w,
+                              // nw = half / groups, bit 8 b + g = replica b of the quad at class rank wi + g nw
+    int32_t split;            // resident +-1 runs: the job runs on the kernel of split words (EaKernel)
+    int32_t threads;          // resident +-1 runs: threads of the CTA that take words (EaBitsShape)
+    double* E_out[2];         // resident +-1 runs: energies of the final and the best states [R], counted
+                              // from the states by the tile itself
 };
 
 // Tile code of the resident kernels (chosen on the host, so the kernel
-// branches on one word of the work item).
+// branches on one word of the work item).  FP32 tiles:
 enum EaTilePath : int32_t {
-    kEaPathFieldsGeneric = 0,  // +-1 couplings with integer fields: generic tile
-    kEaPathFast32 = 1,         // compile-time tile L = 32, WT = 1
-    kEaPathFast16 = 2,         // L = 16, WT = 4
-    kEaPathFast8 = 3,          // L = 8, WT = 16
-    kEaPathGeneric = 4,        // any other even L <= 32
-    kEaPathGen12 = 6,          // generic tile with compile-time L = 12, WT = 4 (+-1 kernel; FP32: generic)
-    kEaPathFast24 = 7,         // compile-time tile L = 24, WT = 1 (576 of the CTA's threads hold sites)
+    kEaPathGeneric = 0,  // any even L <= 32
+    kEaPathFast32 = 1,   // compile-time tile L = 32, WT = 1
+    kEaPathFast16 = 2,   // L = 16, WT = 4
+    kEaPathFast8 = 3,    // L = 8, WT = 16
+    kEaPathFast24 = 7,   // compile-time tile L = 24, WT = 1 (576 of the CTA's threads hold sites)
 };
+
+// +-1 tiles (ea_bits.cuh): G sites per spin word, CPT Philox calls of a word per
+// thread, the thread's words all in one (x, y) column or not, with fields or not.
+__host__ __device__ constexpr int32_t ea_bits_path(int G, int CPT, bool column, bool has_h)
+{
+    return (1 << 16) | (G << 8) | (CPT << 4) | (column ? 2 : 0) | (has_h ? 1 : 0);
+}
+// Sites per spin word of a +-1 tile: gcd(L, 8) for an even L.
+__host__ __device__ constexpr int ea_bits_groups(int L) { return L % 8 == 0 ? 8 : (L % 4 == 0 ? 4 : 2); }
 
 struct EaWork {
     int32_t job;
     int32_t tile;
-    int32_t path;  // EaTilePath of the job
+    int32_t path;  // EaTilePath, or ea_bits_path of a +-1 job
 };
+
+// Shared memory of one +-1 tile: byte offsets of its parts.  Spins: two buffers of
+// class 0, one of class 1, then the best state; bond words and field bytes; two
+// threshold rows (with fields); two sets of energy sums; improved flags.
+struct EaBitsLayout {
+    size_t best, bonds, h, tab, eacc, flags, total;
+    int tab_bytes;  // of one row
+};
+
+__host__ __device__ inline EaBitsLayout ea_bits_layout(int L, int WT, int has_h, int nF)
+{
+    const size_t N = (size_t)L * L * L;
+    const int G = ea_bits_groups(L);
+    const size_t words = N / 2 / G * WT;  // of one class
+    EaBitsLayout o{};
+    size_t b = 3 * words * 4;
+    o.best = b;
+    b += 2 * words * 4;
+    b = (b + 15) / 16 * 16;
+    o.bonds = b;
+    b += N / G * (G == 8 ? 8 : 4);
+    o.h = b;
+    if (has_h) b += N;
+    b = (b + 15) / 16 * 16;
+    o.tab = b;
+    o.tab_bytes = has_h ? (nF + 3) / 4 * 16 : 0;
+    b += 2 * (size_t)o.tab_bytes;
+    o.eacc = b;
+    b += 2 * (size_t)4 * WT * 4;
+    o.flags = b;
+    b += (size_t)4 * WT;
+    o.total = (b + 127) / 128 * 128;
+    return o;
+}
+
+// CTA of the +-1 kernel: 512 threads of 128 registers.  With 1024 threads of 64 the
+// tiles ran 7% (L = 32) to 35% (L = 16, one quad) slower, with 256 threads 8% slower
+// at L = 32 (too few warps).
+constexpr int kBitsThreads = 512;
+
+// Launch shape of a +-1 tile of the job.
+struct EaBitsShape {
+    int lanes;    // threads per spin word
+    int threads;  // of the CTA that the tile keeps busy, whole warps
+    bool column;  // a thread's words are in one (x, y) column
+};
+// One thread per word shares the word's neighbour loads and counts among all its G
+// Philox calls.  Tiles of fewer than 256 words (8 warps) are bound by latency, not by
+// the SM's pipes: with `split`, the calls of a word go to threads of their own, lanes of
+// one word staying inside a warp (L = 6, 64 replicas: 0.9 against 1.2 us per sweep; at
+// 256 words, L = 16, splitting lost 12%).
+inline EaBitsShape ea_bits_shape(const EaJob& j, bool split)
+{
+    const int G = ea_bits_groups(j.inst.L);
+    const int words = j.inst.N / 2 / G * j.WT;  // of one class
+    EaBitsShape o{1, 0, false};
+    while (split && 2 * o.lanes <= G && words * 2 * o.lanes <= kBitsThreads && words * o.lanes < 256 &&
+           2 * o.lanes * j.WT <= 32)
+        o.lanes *= 2;
+    if (j.inst.has_h && o.lanes > 1)  // compiled with fields: one thread per word or one per call
+        o.lanes = G * j.WT <= 32 && words * G <= kBitsThreads ? G : 1;
+    // (Fewer threads with even shares of the words ran slower: L = 24 by 12%, as 14 warps load the four
+    // schedulers of an SM unevenly.)
+    const int need = words * o.lanes;
+    o.threads = need >= kBitsThreads ? kBitsThreads : need < 128 ? 128 : (need + 31) / 32 * 32;
+    const int columns = j.inst.L / 2 * j.inst.L * j.WT;
+    o.column = need <= o.threads || (o.threads / o.lanes) % columns == 0;
+    return o;
+}
 
 inline int32_t ea_tile_path(const EaJob& j)
 {
-    if (j.inst.jtype == PB_J_PM1_I8 && j.inst.has_h) return kEaPathFieldsGeneric;
+    if (j.inst.jtype == PB_J_PM1_I8) {
+        const EaBitsShape o = ea_bits_shape(j, j.split != 0);
+        const int G = ea_bits_groups(j.inst.L), cpt = G / o.lanes;
+        // compiled variants: one thread per word with fields has no column form, several have only that
+        const bool column = cpt < G ? true : (j.inst.has_h ? false : o.column);
+        return ea_bits_path(G, cpt, column, j.inst.has_h != 0);
+    }
     if (j.inst.L == 32 && j.WT == 1) return kEaPathFast32;
     if (j.inst.L == 16 && j.WT == 4) return kEaPathFast16;
     if (j.inst.L == 8 && j.WT == 16) return kEaPathFast8;
     if (j.inst.L == 24 && j.WT == 1) return kEaPathFast24;
-    if (j.inst.L == 12 && j.WT == 4) return kEaPathGen12;
     return kEaPathGeneric;
 }
 
-// Persistent resident kernels: one for +-1 couplings and two for FP32, which
+inline int ea_tile_threads(const EaJob& j)
+{
+    return j.inst.jtype == PB_J_PM1_I8 ? ea_bits_shape(j, j.split != 0).threads : 1024;
+}
+
+// Persistent resident kernels.  For +-1 couplings, one with a thread per spin word
+// and one with several (a launch takes the second if all its +-1 tiles gain by it;
+// with both forms in one kernel, their shared register allocation spilled 230 B a
+// thread and L = 32 ran 6% slower).  Two for FP32, which
 // differ in their compile-time tiles -- the L = 32 tile, or the L = 24 tile,
 // beside L = 16, L = 8 and the runtime-shaped generic tile.  With both the
 // L = 32 and the L = 24 tile in one kernel, the register allocation they share
 // slowed the L = 32 tile by 8%.  A batch takes the L = 24 kernel when its FP32
 // tiles include L = 24 ones and no L = 32 ones; otherwise L = 24 FP32 tiles
 // run the generic tile of the first kernel.
-enum EaKernel : int32_t { kEaKernelPm1 = 0, kEaKernelF32 = 1, kEaKernelF32L24 = 2, kEaKernels = 3 };
+enum EaKernel : int32_t {
+    kEaKernelPm1 = 0,
+    kEaKernelPm1Split = 1,
+    kEaKernelF32 = 2,
+    kEaKernelF32L24 = 3,
+    kEaKernels = 4
+};
+// The +-1 kernel of a launch: split words if every +-1 job of it has tiles that gain.
+inline bool ea_bits_gains_by_split(const EaJob& j) { return ea_bits_shape(j, true).lanes > 1; }
 
 // Shared memory of one resident tile, in bytes.
 __host__ __device__ inline size_t ea_resident_smem(int L, int WT, int jtype, int has_h, int nF)
 {
+    if (jtype == PB_J_PM1_I8) return ea_bits_layout(L, WT, has_h, nF).total;
     const size_t N = (size_t)L * L * L;
-    size_t b = N * (size_t)WT * 4;                       // spins [2][half][WT]
-    if (jtype == PB_J_PM1_I8) {
-        b += (N + 15) / 16 * 16;                         // bond-sign bytes [2][half]
-        if (has_h) b += (N + 15) / 16 * 16;              // h bytes
-    }
-    const int tabw = (jtype == PB_J_PM1_I8) ? (has_h ? nF : 64) : 0;
-    b += (size_t)2 * ((tabw + 3) / 4 * 4) * 4;           // double-buffered threshold row
-    b += (size_t)(1024 / 32) * 4 * WT * 4;               // per-warp energy partials
-    if (jtype == PB_J_PM1_I8 && has_h) b += (size_t)(1024 / 32) * 4 * WT * 4;  // per-warp h.m partials
-    b += (size_t)4 * WT;                                 // improved flags
-    // compile-time-shaped tiles keep their bond bytes as [2][L/8][threads] words
-    const bool fast =
-        !has_h && ((L == 32 && WT == 1) || (L == 16 && WT == 4) || (L == 8 && WT == 16) || (L == 24 && WT == 1));
-    if (fast && jtype == PB_J_PM1_I8) {
-        const size_t f = N * (size_t)WT * 4 + (size_t)(1024 / 32) * 4 * WT * 4 + 128 + (size_t)2 * (L / 8) * 1024 * 4;
-        if (f > b) b = f;
-    }
+    size_t b = N * (size_t)WT * 4;          // spins [2][half][WT]
+    b += (size_t)(1024 / 32) * 4 * WT * 4;  // per-warp energy partials
+    b += (size_t)4 * WT;                    // improved flags
     return (b + 127) / 128 * 128;
 }
 
@@ -116,8 +207,9 @@ cudaError_t ea_resident_set_smem(int kernel, size_t smem);
 // type.  after_previous: programmatic dependent launch on the kernel launched
 // just before it on `st` (its CTAs start as that kernel's CTAs leave; the
 // caller orders any later consumer after both).
+// threads: the largest ea_tile_threads of its jobs.
 cudaError_t ea_launch_resident(int kernel, const EaJob* d_jobs, const EaWork* d_work, int n_work, int* d_counter,
-                               size_t smem, int grid, bool after_previous, cudaStream_t st);
+                               size_t smem, int grid, int threads, bool after_previous, cudaStream_t st);
 // Random-word ceiling: `blocks` CTAs of kResidentThreads threads, each thread drawing the
 // decision words of 32 sites (one L = 32 column, both colours) per sweep; sink holds
 // blocks * kResidentThreads words.  Updates counted: blocks * kResidentThreads * 32 * 4 per sweep.
@@ -125,8 +217,9 @@ cudaError_t ea_launch_philox_ceiling(uint64_t seed, int sweeps, int blocks, uint
 cudaError_t ea_launch_plain_init(const EaJob& job, cudaStream_t st);
 cudaError_t ea_launch_plain_sweep(const EaJob& job, int s, cudaStream_t st);
 cudaError_t ea_launch_plain_energy(const EaJob& job, int s, bool init, cudaStream_t st);
-// Tile layout -> [R][N] int8 +-1, and energies recomputed from those states
-// (int64 for PM1, FP64 for F32).
+// State buffer -> [R][N] int8 +-1, and energies recomputed from those states
+// (int64 for PM1, FP64 for F32; not where job.groups is set: the resident +-1
+// tiles have written E_out themselves).
 cudaError_t ea_launch_readout(const EaJob& job, const uint32_t* words, int8_t* out_pm, double* out_E,
                               cudaStream_t st);
 cudaError_t ea_launch_fields(const EaDevice& inst, const int8_t* d_states, int R, float* d_out, cudaStream_t st);

@@ -341,7 +341,9 @@ pb_status ea_prepare_run(pb_run* run, pb_instance* I, const pb_schedule* sc, int
         j.n_tiles = (Rw + WT - 1) / WT;
     }
     const int Rpad = j.n_tiles * 4 * j.WT;
-    const size_t words = (size_t)j.n_tiles * I->N * j.WT;
+    // resident +-1 runs keep one bit per spin
+    j.groups = form != PB_FORM_PLAIN && I->jtype == PB_J_PM1_I8 ? ea_bits_groups(I->L) : 0;
+    const size_t words = (size_t)j.n_tiles * (I->N / std::max(1, j.groups)) * j.WT;
     const int nlev = std::max<int>(1, (int)betas.size());
     if (I->jtype == PB_J_PM1_I8) {
         const int fmax = 6 + I->hmax;
@@ -393,6 +395,8 @@ pb_status ea_prepare_run(pb_run* run, pb_instance* I, const pb_schedule* sc, int
     PB_ALLOC(run->best_pm, (size_t)R * I->N);
     PB_ALLOC(run->final_pm, (size_t)R * I->N);
     PB_ALLOC(run->E_out, (size_t)2 * R * 8);
+    j.E_out[0] = run->E_out.as<double>();
+    j.E_out[1] = run->E_out.as<double>() + R;
     PB_CUDA_TRY(cudaEventCreate(&run->ev_start));
     PB_CUDA_TRY(cudaEventCreate(&run->ev_stop));
     return PB_OK;
@@ -451,14 +455,20 @@ pb_status ea_batch_setup(std::vector<pb_run*>& runs, cudaStream_t st, std::share
         f32_l24 |= ea_tile_path(r->job) == kEaPathFast24;
         f32_l32 |= ea_tile_path(r->job) == kEaPathFast32;
     }
-    grp[0].kernel = kEaKernelPm1;
+    bool split = true;
+    for (const pb_run* r : runs)
+        if (r->job.inst.jtype == PB_J_PM1_I8) split &= ea_bits_gains_by_split(r->job);
+    grp[0].kernel = split ? kEaKernelPm1Split : kEaKernelPm1;
     grp[1].kernel = f32_l24 && !f32_l32 ? kEaKernelF32L24 : kEaKernelF32;
     for (size_t q = 0; q < runs.size(); ++q) {
-        const EaJob& j = runs[q]->job;
+        EaJob& j = runs[q]->job;
+        j.split = split ? 1 : 0;
+        j.threads = ea_tile_threads(j);
         jobs.push_back(j);
         const int t = j.inst.jtype == PB_J_F32 ? 1 : 0;
         grp[t].smem = std::max(grp[t].smem, ea_resident_smem(j.inst.L, j.WT, j.inst.jtype, j.inst.has_h, j.nF));
-        const double per = (double)j.inst.N * 4.0 * j.WT * std::max(1, j.S) * (t ? 1.8 : 1.0);
+        grp[t].threads = std::max(grp[t].threads, ea_tile_threads(j));
+        const double per = (double)j.inst.N * 4.0 * j.WT * std::max(1, j.S) * (t ? 2.0 : 1.0);
         for (int k = 0; k < j.n_tiles; ++k) tiles[t].push_back({(int)q, k, per});
         grp[t].cost += per * j.n_tiles;
         grp[t].longest = std::max(grp[t].longest, per);
@@ -529,7 +539,7 @@ pb_status ea_batch_launch(std::vector<pb_run*>& runs, const std::shared_ptr<Batc
         for (size_t k = 0; k < shared->groups.size(); ++k) {
             const EaGroup& g = shared->groups[k];
             PB_CUDA_TRY(ea_launch_resident(g.kernel, shared->jobs.as<EaJob>(), shared->work.as<EaWork>() + g.offset, g.n,
-                                           shared->counter.as<int>() + k, g.smem, g.grid, capture && k > 0, st));
+                                           shared->counter.as<int>() + k, g.smem, g.grid, g.threads, capture && k > 0, st));
             if (capture) PB_CUDA_TRY(cudaEventRecord(shared->ev_group[k], st));
         }
         if (capture)
@@ -742,19 +752,21 @@ static pb_status ea_anneal_resume(pb_instance* I, const pb_schedule* sc, int32_t
     EaJob& j = run->job;
     const bool pm1 = I->jtype == PB_J_PM1_I8;
     const int64_t N = I->N, half = N / 2, L = I->L, Rpad = (int64_t)j.n_tiles * 4 * j.WT;
-    // [R][N] +-1 -> tile layout: word ((tile * 2 + c) * half + k) * WT + w, byte b of replica
-    // r = (tile * WT + w) * 4 + b; +-1: bit 8b set <=> m = -1; FP32: byte 0x3F / 0xBF; padding replicas +1
+    // [R][N] +-1 -> tile layout of replica r = (tile * WT + w) * 4 + b.  FP32: word ((tile * 2 + c) * half + k)
+    // * WT + w, byte b 0x3F / 0xBF; +-1: word ((tile * 2 + c) * nw + k % nw) * WT + w, bit 8b + k / nw set
+    // <=> m = -1.  Padding replicas +1.
+    const int64_t G = pm1 ? j.groups : 1, nw = half / G;
     const uint32_t fill = pm1 ? 0u : 0x3F3F3F3Fu;
-    std::vector<uint32_t> w((size_t)(Rpad / 4 * N), fill), wb((size_t)(Rpad / 4 * N), fill);
+    std::vector<uint32_t> w((size_t)(Rpad / 4 * (N / G)), fill), wb((size_t)(Rpad / 4 * (N / G)), fill);
     for (int64_t r = 0; r < R; ++r) {
         const int64_t tile = r / (4 * j.WT), ww = (r / 4) % j.WT, b = r & 3;
-        const uint32_t bit = pm1 ? (1u << (8 * b)) : (0x80u << (8 * b));
         for (int64_t i = 0; i < N; ++i) {
             const int8_t m = state[r * N + i], mb = best_state[r * N + i];
             if ((m != 1 && m != -1) || (mb != 1 && mb != -1)) return fail(PB_EINVAL, "states must hold +1 or -1");
             const int64_t x = i % L, y = (i / L) % L, z = i / (L * L);
             const int64_t c = (x + y + z) & 1, k = i >> 1;
-            const size_t idx = (size_t)(((tile * 2 + c) * half + k) * j.WT + ww);
+            const size_t idx = (size_t)(((tile * 2 + c) * nw + k % nw) * j.WT + ww);
+            const uint32_t bit = pm1 ? (1u << (8 * b + k / nw)) : (0x80u << (8 * b));
             if (m < 0) w[idx] |= bit;
             if (mb < 0) wb[idx] |= bit;
         }

@@ -123,7 +123,8 @@ extern "C" pb_status pb_anneal_ea_noalloc(int32_t L, const int8_t* J_dev, const 
     const int Rpad = n_tiles * 4 * WT;
     const int nlev = std::max<int>(1, (int)betas.size());
 
-    // scratch layout
+    // scratch layout; the two state sets are given one byte per spin, the size the call's
+    // documented limit counts, though the tiles need one bit
     size_t off = 0;
     const size_t o_job = off;      off = align256(off + sizeof(EaJob));
     const size_t o_work = off;     off = align256(off + (size_t)n_tiles * sizeof(EaWork));
@@ -164,8 +165,13 @@ extern "C" pb_status pb_anneal_ea_noalloc(int32_t L, const int8_t* J_dev, const 
     j.fmin = fmin;
     j.table = reinterpret_cast<const uint32_t*>(S + o_tab);
     j.R = replicas;
+    j.groups = ea_bits_groups(L);
+    j.E_out[0] = final_E_dev;
+    j.E_out[1] = best_E_dev;
     j.WT = WT;
     j.n_tiles = n_tiles;
+    j.split = ea_bits_gains_by_split(j) ? 1 : 0;
+    j.threads = ea_tile_threads(j);
     j.best_words = reinterpret_cast<uint32_t*>(S + o_best);
     j.final_words = reinterpret_cast<uint32_t*>(S + o_final);
     j.E_best_i = reinterpret_cast<int32_t*>(S + o_E);
@@ -185,10 +191,11 @@ extern "C" pb_status pb_anneal_ea_noalloc(int32_t L, const int8_t* J_dev, const 
     PB_CUDA_TRY(cudaGetLastError());
 
     const size_t smem = ea_resident_smem(L, WT, PB_J_PM1_I8, 0, nF);
-    PB_CUDA_TRY(ea_resident_set_smem(kEaKernelPm1, smem));
-    PB_CUDA_TRY(ea_launch_resident(kEaKernelPm1, reinterpret_cast<const EaJob*>(S + o_job),
+    const int kernel = j.split ? kEaKernelPm1Split : kEaKernelPm1;
+    PB_CUDA_TRY(ea_resident_set_smem(kernel, smem));
+    PB_CUDA_TRY(ea_launch_resident(kernel, reinterpret_cast<const EaJob*>(S + o_job),
                                    reinterpret_cast<const EaWork*>(S + o_work), n_tiles, reinterpret_cast<int*>(S + o_ctr),
-                                   smem, std::min(n_tiles, sms), false, st));
+                                   smem, std::min(n_tiles, sms), ea_tile_threads(j), false, st));
     PB_CUDA_TRY(ea_launch_readout(j, j.final_words, final_states_dev, final_E_dev, st));
     PB_CUDA_TRY(ea_launch_readout(j, j.best_words, best_states_dev, best_E_dev, st));
     PB_CUDA_TRY(cudaMemcpyAsync(best_sweep_dev, j.best_sweep, (size_t)replicas * 4, cudaMemcpyDeviceToDevice, st));
