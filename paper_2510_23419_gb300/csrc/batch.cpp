@@ -90,8 +90,13 @@ double est_cost(const pb_instance* I, int R, int S, int form, double* compute = 
         lat = 3.0 * std::max(1, S) * 2e-6;
     } else {
         const double flop = upd * 2.0 * I->n * (I->jtype == PB_J_F32 ? 2.0 : 1.0);
-        if (form == PB_FORM_RESIDENT) {  // one CTA per 32 replicas: ~8 us per sweep at n = 256 (+-1), FP32 ~4x slower
-            c = std::max(1, S) * 8e-6 * (I->n / 256.0) * (I->n / 256.0) * (I->jtype == PB_J_F32 ? 4.0 : 1.0);
+        if (form == PB_FORM_RESIDENT) {
+            // latency-bound: a sweep takes about the same time whatever the replicas (up to 8 quads per CTA)
+            const int sms = sm_count(), g = bq_res_groups(R, false, sms), ctas = ((R + 3) / 4 + g - 1) / g;
+            const double sweep = I->jtype == PB_J_F32 ? 0.6e-6 + 15e-9 * I->n * (1.0 + 0.35 * (g - 1))
+                                                      : 0.5e-6 + 3e-9 * I->n * (1.0 + 0.15 * (g - 1));
+            c = std::max(1, S) * sweep * ctas / sms;
+            lat = std::max(1, S) * sweep;
         } else {
             const double rate = form == PB_FORM_CUDACORE ? 2.5e13 : (I->jtype == PB_J_F32 ? 1.5e15 : 1.8e15);
             // small instances fill a fraction of the tensor tiles
@@ -508,7 +513,7 @@ pb_status pb_autotune(pb_instance* I, int32_t R, int32_t probe_sweeps, void* str
                 units = std::min(sms, 2 * bq_tc_clusters(I->n, run->bjob.Rpad, I->jtype == PB_J_PM1_I8 ? 0 : 1,
                                                          wt != 0));
             } else if (form == PB_FORM_RESIDENT) {
-                units = std::min(sms, (R + 31) / 32);
+                units = std::min(sms, ((R + 3) / 4 + run->res_groups - 1) / run->res_groups);
             } else {
                 units = std::min(sms, ((I->n + 63) / 64) * ((R + 63) / 64));
             }

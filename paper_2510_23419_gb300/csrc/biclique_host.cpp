@@ -173,7 +173,7 @@ bool bq_resident_fits(const pb_instance* I)
     if (I->topo != PB_TOPO_BICLIQUE || I->n > nmax) return false;
     // the widest threshold window is at most the whole row (2 (n + |h|) + 1 entries)
     const int tab = I->jtype == PB_J_PM1_I8 ? 2 * (I->n + I->hmax) + 1 : 0;
-    return bq_res_smem_bytes(I->jtype, I->n, tab) <= 227 * 1024;
+    return bq_res_smem_bytes(I->jtype, I->n, kBqResReps / 4, tab) <= 227 * 1024;
 }
 
 static pb_status bq_prepare(pb_run* run, pb_instance* I, const pb_schedule* sc, int R, uint64_t seed,
@@ -304,8 +304,9 @@ static pb_status bq_prepare(pb_run* run, pb_instance* I, const pb_schedule* sc, 
         j.pdl = bq_tc_fills_device(n, j.Rpad, pm1 ? 0 : 1) ? 1 : 0;
     }
     if (resident) {
-        run->res_smem = bq_res_smem_bytes(I->jtype, n, pm1 ? run->res_tab : 0);
-        PB_CUDA_TRY(bq_res_set_smem(I->jtype, run->res_smem));
+        run->res_groups = bq_res_groups(R, j.has_target == 2, sm_count());
+        run->res_smem = bq_res_smem_bytes(I->jtype, n, run->res_groups, pm1 ? run->res_tab : 0);
+        PB_CUDA_TRY(bq_res_set_smem(I->jtype, n, run->res_smem));
     }
     PB_CUDA_TRY(cudaEventCreate(&run->ev_start));
     PB_CUDA_TRY(cudaEventCreate(&run->ev_stop));
@@ -399,7 +400,7 @@ static pb_status bq_launch_resident(pb_run* run, cudaStream_t st)
     const BqJob& j = run->bjob;
     PB_CUDA_TRY(cudaEventRecord(run->ev_start, st));
     PB_CUDA_TRY(cudaEventRecord(run->ev_k0, st));
-    PB_CUDA_TRY(bq_launch_res(j, j.inst.jtype == PB_J_PM1_I8 ? run->res_tab : 0, run->res_smem, st));
+    PB_CUDA_TRY(bq_launch_res(j, run->res_groups, j.inst.jtype == PB_J_PM1_I8 ? run->res_tab : 0, run->res_smem, st));
     PB_CUDA_TRY(cudaEventRecord(run->ev_k1, st));
     const int last = (j.S - 1) & 1;
     PB_CUDA_TRY(bq_launch_readout(bq_view(j, 0, last, last), 0, run->final_pm.as<int8_t>(), run->E_out.as<double>(), st));

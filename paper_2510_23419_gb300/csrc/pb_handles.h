@@ -145,6 +145,7 @@ struct pb_run {
     pb::DevBuf bq_alt[2];  // biclique: the parity-1 live spin buffers of sides A and B
     std::vector<int32_t> csr_nchunk;  // general graph: class chunks of each colour class
     int res_tab = 0;                  // biclique resident form: widest threshold window
+    int res_groups = 0;               // biclique resident form: quads of replicas per CTA
     size_t res_smem = 0;              // biclique resident form: dynamic shared memory per CTA
     std::vector<int32_t> bq_win;  // biclique +-1: per beta level, (first index, width, offset) of its threshold window
     std::shared_ptr<pb::BatchShared> batch;
