@@ -90,7 +90,7 @@ double est_cost(const pb_instance* I, int R, int S, int form, double* compute = 
         lat = 3.0 * std::max(1, S) * 2e-6;
     } else {
         const double flop = upd * 2.0 * I->n * (I->jtype == PB_J_F32 ? 2.0 : 1.0);
-        if (form == PB_FORM_RESIDENT) {
+        if (form == PB_FORM_RESIDENT || form == kFormResidentWide) {
             // latency-bound: a sweep takes about the same time whatever the replicas (up to 8 quads per CTA)
             const int sms = sm_count(), g = bq_res_groups(R, false, sms), ctas = ((R + 3) / 4 + g - 1) / g;
             const double sweep = I->jtype == PB_J_F32 ? 0.6e-6 + 15e-9 * I->n * (1.0 + 0.35 * (g - 1))
@@ -120,9 +120,9 @@ struct Job {
 }  // namespace
 
 // Form and tile width the library picks for a job whose caller left the form open.
-void choose_form(const pb_instance* I, int R, int requested, int& form, int& wt)
+void choose_form(const pb_instance* I, int R, int requested, int& form, int& wt, const pb_anneal_opts* opts)
 {
-    form = requested;
+    form = requested == kFormResidentWide ? -1 : requested;  // not a form a caller can name
     wt = 0;
     TuneEntry te;
     const bool tuned = requested == PB_FORM_AUTO && tune_lookup(I, R, te);
@@ -152,7 +152,10 @@ void choose_form(const pb_instance* I, int R, int requested, int& form, int& wt)
             wt = te.wt;
         }
         // small instances: the resident form (no launch per half-sweep); else tensor cores
-        if (form == PB_FORM_AUTO) form = bq_resident_fits(I) ? PB_FORM_RESIDENT : PB_FORM_TENSOR;
+        if (form == PB_FORM_AUTO) {
+            const bool wide = bq_resident_wide(I, R) && !(opts && opts->flags != 0);
+            form = bq_resident_fits(I) ? PB_FORM_RESIDENT : wide ? kFormResidentWide : PB_FORM_TENSOR;
+        }
     }
 }
 
@@ -213,14 +216,14 @@ pb_status batch_start(int count, pb_instance* const* insts, const pb_schedule* s
         if (!I) return fail(PB_EINVAL, "null instance in batch");
         if (replicas[q] < 1) return fail(PB_EINVAL, "replicas must be >= 1");
         int form = 0, wt = 0;
-        choose_form(I, replicas[q], opts ? opts[q].form : PB_FORM_AUTO, form, wt);
+        choose_form(I, replicas[q], opts ? opts[q].form : PB_FORM_AUTO, form, wt, opts ? &opts[q] : nullptr);
         if (I->topo == PB_TOPO_EA3D) {
             if (form == PB_FORM_RESIDENT && wt == 0) return fail(PB_EUNSUPPORTED, "lattice too large for the resident form");
             if (form != PB_FORM_RESIDENT && form != PB_FORM_PLAIN)
                 return fail(PB_EUNSUPPORTED, "form not available for EA instances");
         } else if (I->topo == PB_TOPO_CSR) {
             if (form != PB_FORM_PLAIN) return fail(PB_EUNSUPPORTED, "general sparse instances run in the plain form");
-        } else if (form != PB_FORM_TENSOR && form != PB_FORM_CUDACORE && form != PB_FORM_RESIDENT) {
+        } else if (form != PB_FORM_TENSOR && form != PB_FORM_CUDACORE && form != PB_FORM_RESIDENT && form != kFormResidentWide) {
             return fail(PB_EUNSUPPORTED, "form not available for biclique instances");
         }
         jobs.push_back(Job{q, I, replicas[q], scheds[q].n_sweeps, form, wt, est_cost(I, replicas[q], scheds[q].n_sweeps, form)});

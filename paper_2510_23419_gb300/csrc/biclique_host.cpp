@@ -176,6 +176,15 @@ bool bq_resident_fits(const pb_instance* I)
     return bq_res_smem_bytes(I->jtype, I->n, kBqResReps / 4, tab) <= 227 * 1024;
 }
 
+// +-1 bicliques past the size a caller may ask the resident form for, where it is still the faster
+// one (us per sweep, resident / tensor: n = 512, 256 replicas 3.6 / 23.8; 4096 replicas
+// 22.1 / 25.8): while its CTAs, of at most 8 quads, fit the SMs in one wave.
+bool bq_resident_wide(const pb_instance* I, int R)
+{
+    return I->topo == PB_TOPO_BICLIQUE && I->jtype == PB_J_PM1_I8 && I->n <= kBqResWideN &&
+           (R + 3) / 4 <= (kBqResReps / 4) * (long long)sm_count();
+}
+
 static pb_status bq_prepare(pb_run* run, pb_instance* I, const pb_schedule* sc, int R, uint64_t seed,
                             const pb_anneal_opts* opts, int form, int tile_split, cudaStream_t st)
 {
@@ -382,6 +391,7 @@ pb_status bq_setup(pb_run* run, pb_instance* I, const pb_schedule* sc, int R, ui
 {
     int form = opts ? opts->form : PB_FORM_AUTO;
     if (form == PB_FORM_AUTO) form = PB_FORM_TENSOR;
+    if (form == kFormResidentWide) return bq_prepare(run, I, sc, R, seed, opts, PB_FORM_RESIDENT, tile_split, st);
     if (form != PB_FORM_TENSOR && form != PB_FORM_CUDACORE && form != PB_FORM_RESIDENT)
         return fail(PB_EUNSUPPORTED, "form not available for biclique instances");
     if (form == PB_FORM_RESIDENT && !bq_resident_fits(I))

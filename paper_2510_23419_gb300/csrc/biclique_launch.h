@@ -67,7 +67,8 @@ constexpr uint64_t kBqWaitNs = 1000000000ull;   // 1 s: far above any tile's MMA
 constexpr uint64_t kBqTestWaitNs = 2000000ull;  // 2 ms: the limit under PB_FLAG_TEST_EXPIRE_WAITS
 
 constexpr int kBqResReps = 32;      // resident form: replica padding (most replicas per CTA)
-constexpr int kBqResMaxNpm1 = 256;  // resident form: largest n (+-1 couplings)
+constexpr int kBqResMaxNpm1 = 256;  // resident form on request: largest n (+-1 couplings)
+constexpr int kBqResWideN = 512;    // resident form chosen by the library: largest n (+-1 couplings)
 constexpr int kBqResMaxNf32 = 128;  // resident form: largest n (real couplings, FP32 J in shared memory)
 
 constexpr int kBqTileRows = 64;   // CUDA-core field kernel: rows (spins of the updated side) per block

@@ -6,8 +6,8 @@
 // two half-sweeps are separated by CTA barriers, and the energy, running best
 // and best-state copies happen in the same launch.
 //
-//  +-1 couplings (n <= 256): one bit per spin and per coupling.  A thread owns row
-//      i of both sides and keeps their coupling signs in registers (8 + 8
+//  +-1 couplings (n <= 512): one bit per spin and per coupling.  A thread owns row
+//      i of both sides and keeps their coupling signs in registers (16 + 16
 //      words at most); F = n - 2 popc(J ^ m) over the row, carry-save
 //      compressed before the population counts; the 32 decisions of a warp are
 //      one ballot, which is the spin word the other side reads.
@@ -94,16 +94,39 @@ __host__ __device__ inline ResLayout res_layout(int jtype, int n, int groups, in
 __device__ __forceinline__ uint8_t enc_byte(bool minus) { return minus ? kE4m3Minus : kE4m3Plus; }
 __device__ __forceinline__ uint16_t enc_half(bool minus) { return minus ? kBf16Minus : kBf16Plus; }
 
-// Set bits of NW words x (carry-save compressed: four population counts for eight words).
+// Full adder of three words, bit by bit: sum s, carry c.
+__device__ __forceinline__ void csa(uint32_t a, uint32_t b, uint32_t d, uint32_t& s, uint32_t& c)
+{
+    s = a ^ b ^ d;
+    c = (a & b) | (d & (a | b));
+}
+// Seven words as bit counts o + 2 t + 4 f.
+__device__ __forceinline__ void csa7(const uint32_t* x, uint32_t& o, uint32_t& t, uint32_t& f)
+{
+    uint32_t s1, c1, s2, c2, c3;
+    csa(x[0], x[1], x[2], s1, c1);
+    csa(x[3], x[4], x[5], s2, c2);
+    csa(s1, s2, x[6], o, c3);
+    csa(c1, c2, c3, t, f);
+}
+
+// Set bits of NW words x, carry-save compressed: four population counts (which run at
+// a quarter of the other instructions' rate) for eight words, five for sixteen.
 template <int NW>
 __device__ __forceinline__ int popc_words(const uint32_t (&x)[NW])
 {
     if constexpr (NW == 8) {
-        const uint32_t s1 = x[0] ^ x[1] ^ x[2], c1 = (x[0] & x[1]) | (x[2] & (x[0] | x[1]));
-        const uint32_t s2 = x[3] ^ x[4] ^ x[5], c2 = (x[3] & x[4]) | (x[5] & (x[3] | x[4]));
-        const uint32_t s3 = s1 ^ s2 ^ x[6], c3 = (s1 & s2) | (x[6] & (s1 | s2));
-        const uint32_t s4 = c1 ^ c2 ^ c3, c4 = (c1 & c2) | (c3 & (c1 | c2));
-        return __popc(s3) + __popc(x[7]) + 2 * __popc(s4) + 4 * __popc(c4);
+        uint32_t o, t, f;
+        csa7(x, o, t, f);
+        return __popc(o) + __popc(x[7]) + 2 * __popc(t) + 4 * __popc(f);
+    } else if constexpr (NW == 16) {
+        uint32_t o1, t1, f1, o2, t2, f2, o, t, f, c, e;
+        csa7(x, o1, t1, f1);
+        csa7(x + 7, o2, t2, f2);
+        csa(o1, o2, x[14], o, c);
+        csa(t1, t2, c, t, c);
+        csa(f1, f2, c, f, e);
+        return __popc(o) + __popc(x[15]) + 2 * __popc(t) + 4 * __popc(f) + 8 * __popc(e);
     } else {
         int t = 0;
 #pragma unroll
@@ -116,7 +139,7 @@ __device__ __forceinline__ void main_barrier(int threads) { asm volatile("bar.sy
 
 // Threads [0, rows * tg) own rows, rows = n rounded up to whole warps, thread group
 // grp of tg the quads grp, grp + tg, ... of the CTA's `groups`; the last warp is the
-// service warp.  NW: spin words per side (+-1: 1, 2, 4 or 8; real couplings: unused).
+// service warp.  NW: spin words per side (+-1: 1, 2, 4, 8 or 16; real couplings: unused).
 template <int JT, int NW>
 __global__ void __launch_bounds__(kResThreads, 1) bq_res_kernel(BqJob job, int groups, int tg, int tab_cap)
 {
@@ -207,18 +230,36 @@ __global__ void __launch_bounds__(kResThreads, 1) bq_res_kernel(BqJob job, int g
     auto fields = [&](int side, int par, int g, int (&Fi)[4], float (&Ff)[4]) {
         if constexpr (PM1) {
             const uint4* o = state(par, 1 - side) + g * W;
-            uint32_t x[4][NW];
+            const int h = side == 0 ? iA : iB;
+            if constexpr (NW <= 8) {
+                uint32_t x[4][NW];
 #pragma unroll
-            for (int w = 0; w < NW; ++w) {
-                const uint4 v = w < W ? o[w] : make_uint4(0u, 0u, 0u, 0u);
-                const uint32_t j = side == 0 ? jA[w] : jB[w];
-                x[0][w] = v.x ^ j;
-                x[1][w] = v.y ^ j;
-                x[2][w] = v.z ^ j;
-                x[3][w] = v.w ^ j;
+                for (int w = 0; w < NW; ++w) {
+                    const uint4 v = w < W ? o[w] : make_uint4(0u, 0u, 0u, 0u);
+                    const uint32_t j = side == 0 ? jA[w] : jB[w];
+                    x[0][w] = v.x ^ j;
+                    x[1][w] = v.y ^ j;
+                    x[2][w] = v.z ^ j;
+                    x[3][w] = v.w ^ j;
+                }
+#pragma unroll
+                for (int k = 0; k < 4; ++k) Fi[k] = n - 2 * popc_words<NW>(x[k]) + h;
+            } else {
+                // two replicas at a time: four would take 64 registers
+#pragma unroll
+                for (int k = 0; k < 4; k += 2) {
+                    uint32_t x[2][NW];
+#pragma unroll
+                    for (int w = 0; w < NW; ++w) {
+                        const uint2 v = w < W ? reinterpret_cast<const uint2*>(o + w)[k >> 1] : make_uint2(0u, 0u);
+                        const uint32_t j = side == 0 ? jA[w] : jB[w];
+                        x[0][w] = v.x ^ j;
+                        x[1][w] = v.y ^ j;
+                    }
+                    Fi[k] = n - 2 * popc_words<NW>(x[0]) + h;
+                    Fi[k + 1] = n - 2 * popc_words<NW>(x[1]) + h;
+                }
             }
-#pragma unroll
-            for (int k = 0; k < 4; ++k) Fi[k] = n - 2 * popc_words<NW>(x[k]) + (side == 0 ? iA : iB);
         } else {
             const uint4* o = reinterpret_cast<const uint4*>(state(par, 1 - side) + g * len);
             const float* Jp = side == 0 ? sJ + (live ? i : 0) * kLdJ : sJ + (live ? i : 0);
@@ -501,7 +542,7 @@ cudaError_t res_attr(size_t bytes)
     return cudaFuncSetAttribute(bq_res_kernel<JT, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
-int res_words(int n) { return n <= 32 ? 1 : n <= 64 ? 2 : n <= 128 ? 4 : 8; }
+int res_words(int n) { return n <= 32 ? 1 : n <= 64 ? 2 : n <= 128 ? 4 : n <= 256 ? 8 : 16; }
 
 }  // namespace
 
@@ -522,9 +563,9 @@ int bq_res_groups(int R, bool stop_mode, int sms)
 cudaError_t bq_res_set_smem(int jtype, int n, size_t bytes)
 {
     static std::mutex mu;
-    static size_t current[64][5] = {};
+    static size_t current[64][6] = {};
     const int nw = res_words(n);
-    const int k = jtype != PB_J_PM1_I8 ? 0 : nw == 1 ? 1 : nw == 2 ? 2 : nw == 4 ? 3 : 4;
+    const int k = jtype != PB_J_PM1_I8 ? 0 : nw == 1 ? 1 : nw == 2 ? 2 : nw == 4 ? 3 : nw == 8 ? 4 : 5;
     int dev = 0;
     cudaGetDevice(&dev);
     std::lock_guard<std::mutex> lock(mu);
@@ -534,7 +575,8 @@ cudaError_t bq_res_set_smem(int jtype, int n, size_t bytes)
                           : k == 1 ? res_attr<PB_J_PM1_I8, 1>(bytes)
                           : k == 2 ? res_attr<PB_J_PM1_I8, 2>(bytes)
                           : k == 3 ? res_attr<PB_J_PM1_I8, 4>(bytes)
-                                   : res_attr<PB_J_PM1_I8, 8>(bytes);
+                          : k == 4 ? res_attr<PB_J_PM1_I8, 8>(bytes)
+                                   : res_attr<PB_J_PM1_I8, 16>(bytes);
     if (e == cudaSuccess && cur) *cur = bytes;
     return e;
 }
@@ -553,8 +595,10 @@ cudaError_t bq_launch_res(const BqJob& job, int groups, int tab_cap, size_t smem
         bq_res_kernel<PB_J_PM1_I8, 2><<<grid, threads, smem, st>>>(job, groups, tg, tab_cap);
     else if (res_words(n) == 4)
         bq_res_kernel<PB_J_PM1_I8, 4><<<grid, threads, smem, st>>>(job, groups, tg, tab_cap);
-    else
+    else if (res_words(n) == 8)
         bq_res_kernel<PB_J_PM1_I8, 8><<<grid, threads, smem, st>>>(job, groups, tg, tab_cap);
+    else
+        bq_res_kernel<PB_J_PM1_I8, 16><<<grid, threads, smem, st>>>(job, groups, tg, tab_cap);
     return cudaGetLastError();
 }
 

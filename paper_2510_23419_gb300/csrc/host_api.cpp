@@ -718,7 +718,7 @@ pb_status pb_anneal_ex(pb_instance* I, const pb_schedule* sc, int32_t R, uint64_
         if (ps != PB_OK) return ps;
     } else {
         int f = 0, wt = 0;
-        choose_form(I, R, form, f, wt);
+        choose_form(I, R, form, f, wt, opts);
         pb_anneal_opts o = opts ? *opts : pb_anneal_opts{PB_FORM_AUTO, 0, NAN};
         o.form = f;
         pb_status ps = bq_anneal(run.get(), I, sc, R, seed, &o, st, wt);

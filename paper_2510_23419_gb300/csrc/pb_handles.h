@@ -199,7 +199,12 @@ pb_status wait_run(pb_run* run, int32_t timeout_ms);
 // Form (and EA tile width) for a job: the caller's choice, else the autotuner's
 // table entry for the job's shape, else the built-in rule.
 // wt: EA resident tile width; biclique tensor form: 1 = split a sparse last round of tiles, 0 = whole tiles.
-void choose_form(const pb_instance* I, int R, int requested, int& form, int& wt);
+// opts (may be null): runs that stop at a target or test the failure path keep the forms whose
+// results depend on the form in the documented way.
+void choose_form(const pb_instance* I, int R, int requested, int& form, int& wt, const pb_anneal_opts* opts = nullptr);
+// A form only the library chooses: +-1 bicliques of 256 < n <= 512 in the resident form.
+constexpr int kFormResidentWide = 1000;
+bool bq_resident_wide(const pb_instance* I, int R);
 pb_status batch_start(int count, pb_instance* const* insts, const pb_schedule* scheds, const int32_t* replicas,
                       const uint64_t* seeds, const pb_anneal_opts* opts, cudaStream_t setup_st, bool join,
                       std::vector<double>* load_io, std::vector<std::unique_ptr<pb_run>>& runs_out,
