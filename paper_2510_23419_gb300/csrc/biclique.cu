@@ -8,7 +8,9 @@
 // Philox word of (i, s, r >> 2, side) and writes the new spins.  Fields of
 // +-1 instances are exact integers in FP32 (|F| <= n + |h| < 2^24).
 #include "biclique_launch.h"
+#include "bit_count.cuh"
 #include "ea_kernels.cuh"
+#include "exact_split.cuh"
 
 namespace pb {
 
@@ -340,39 +342,168 @@ __global__ void __launch_bounds__(256) bq_best_flush_kernel(BqJob job)
     bq_copy_flagged(job, r0, s_copy, last & 1);
 }
 
+// Spin words of a state set: bit c of word [r][side][w] set <=> m of spin 32 w + c is -1.
 __global__ void __launch_bounds__(256) bq_readout_kernel(BqJob job, int which, int8_t* __restrict__ out)
 {
-    const int n = job.inst.n;
+    // a thread reads 32 encoded spins and writes their 32 output bytes and, for +-1, their bit word
+    const int n = job.inst.n, W = (n + 31) / 32;
     const long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= (long long)job.R * 2 * n) return;
-    const int r = (int)(j / (2 * n));
-    const int c = (int)(j - (long long)r * 2 * n);
-    const int side = c >= n ? 1 : 0;
-    const int i = c - side * n;
+    if (j >= 2LL * job.R * W) return;
+    const int rs = (int)(j / W), w = (int)(j - (long long)rs * W);
+    const int r = rs >> 1, side = rs & 1;
     const void* src_side;
     if (which)
         src_side = job.best[side];
-    else if (job.has_target == 2 && job.stop[1] >= 0)  // stopped early: the live buffers of that sweep
+    else if (job.has_target == 2 && job.stop && job.stop[1] >= 0)  // stopped early: the live buffers of that sweep
         src_side = job.buf[side][job.stop[1] & 1];
     else
         src_side = job.spins[side];
-    bool minus;
-    if (job.inst.jtype == PB_J_PM1_I8)
-        minus = static_cast<const uint8_t*>(src_side)[(size_t)r * job.ld + i] & 0x80u;
-    else
-        minus = static_cast<const uint16_t*>(src_side)[(size_t)r * job.ld + i] & 0x8000u;
-    out[j] = minus ? (int8_t)-1 : (int8_t)1;
+    const bool pm1 = job.inst.jtype == PB_J_PM1_I8;
+    uint32_t bits = 0;
+    // rows are multiples of 16 elements, so whole 16-byte loads stay inside the row
+    if (pm1) {
+        const uint4* src = reinterpret_cast<const uint4*>(static_cast<const uint8_t*>(src_side) + (size_t)r * job.ld) + 2 * w;
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            if (32 * w + 16 * q >= n) break;
+            const uint4 v = src[q];
+            const uint32_t x[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const uint32_t t = (x[u] >> 7) & 0x01010101u;  // the four sign bits to bits 0..3
+                bits |= ((t | (t >> 7) | (t >> 14) | (t >> 21)) & 0xFu) << (16 * q + 4 * u);
+            }
+        }
+    } else {
+        const uint4* src = reinterpret_cast<const uint4*>(static_cast<const uint16_t*>(src_side) + (size_t)r * job.ld) + 4 * w;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            if (32 * w + 8 * q >= n) break;
+            const uint4 v = src[q];
+            const uint32_t x[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int u = 0; u < 4; ++u) bits |= (((x[u] >> 15) & 1u) | ((x[u] >> 30) & 2u)) << (8 * q + 2 * u);
+        }
+    }
+    const int left = n - 32 * w;
+    if (left < 32) bits &= (1u << left) - 1u;
+    if (pm1) job.sbits[j] = bits;
+    int8_t* dst = out + (size_t)r * 2 * n + (size_t)side * n + 32 * w;
+    if (left >= 32 && (n & 3) == 0) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const uint32_t f = (bits >> (4 * u)) & 0xFu;
+            const uint32_t t = (f & 1u) | ((f & 2u) << 7) | ((f & 4u) << 14) | ((f & 8u) << 21);
+            reinterpret_cast<uint32_t*>(dst)[u] = 0x01010101u + t * 0xFEu;  // 0x01 = +1, 0xFF = -1
+        }
+    } else {
+        for (int c = 0; c < min(left, 32); ++c) dst[c] = ((bits >> c) & 1u) ? (int8_t)-1 : (int8_t)1;
+    }
+}
+
+// Sign words of +-1 couplings: bit c of word [i][w] set <=> J[i][32 w + c] = -1.
+__global__ void __launch_bounds__(256) bq_sign_words_kernel(const int8_t* __restrict__ J, int n, uint32_t* __restrict__ out)
+{
+    const int W = (n + 31) / 32, lane = threadIdx.x & 31;
+    const long long word = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);  // a warp per word
+    if (word >= (long long)n * W) return;
+    const int i = (int)(word / W), j = (int)(word - (long long)i * W) * 32 + lane;
+    const uint32_t m = __ballot_sync(0xFFFFFFFFu, j < n && J[(size_t)i * n + j] < 0);
+    if (lane == 0) out[word] = m;
 }
 
 // Exact energy of returned states (Eq. 1 with the sign reading E = -sum J a b - sum h m).
-// Tiled over 64 rows i x 64 replicas r: U[i][r] = sum_j J[i][j] b[r][j], then
+// Tiled over 64 rows i x 64 replicas r, 4 x 4 per thread: U[i][r] = sum_j J[i][j] b[r][j], then
 // the tile's part -sum_i a[r][i] U[i][r] goes to epart[row tile][r].
-//   +-1: int8 products four at a time (__dp4a), exact int32 (|U| <= n).
-//   real: U as an unevaluated FP32 pair hi + lo, every term added by the
-//         error-free two-sum (Knuth), so U is accurate to about 2^-48
-//         relative to sum_j |J_ij|; the row sum is taken in FP64.
 constexpr int kEt = 64;
+constexpr int kEtLd = kEt + 4;  // row stride in shared memory: vector loads of 4 neighbours, no conflicts
 
+// The tile's -sum_i a U per replica: the threads' rows, then the 16 row quads in order.
+__device__ __forceinline__ void bq_energy_reduce(const BqJob& job, const double (&part)[4], int r0, double (&red)[16][kEt + 1])
+{
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+#pragma unroll
+    for (int b = 0; b < 4; ++b) red[ty][tx * 4 + b] = part[b];
+    __syncthreads();
+    if (threadIdx.x < kEt) {
+        const int r = r0 + threadIdx.x;
+        double t = 0.0;
+        for (int q = 0; q < 16; ++q) t += red[q][threadIdx.x];
+        if (r < job.R) job.epart[(size_t)blockIdx.x * job.R + r] = t;
+    }
+}
+
+// +-1: U = n - 2 popc(J ^ b) on sign words, eight words at a time carry-save compressed to four
+// population counts.  n = 4096, 4096 replicas: 0.64 ms per state set with its state copy (int8
+// products with __dp4a and a byte per thread, which this replaces, 1.79 ms).
+__global__ void __launch_bounds__(256) bq_energy_bits_kernel(BqJob job)
+{
+    const int n = job.inst.n, R = job.R, W = (n + 31) / 32;
+    const int i0 = blockIdx.x * kEt, r0 = blockIdx.y * kEt;
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;  // replica quad, row quad
+    constexpr int KW = 16;                                     // words per stage
+    __shared__ __align__(16) uint32_t Js[KW][kEtLd];
+    __shared__ __align__(16) uint32_t Bs[KW][kEtLd];
+    __shared__ double red[16][kEt + 1];
+    int pc[4][4];
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) pc[a][b] = 0;
+    for (int w0 = 0; w0 < W; w0 += KW) {
+        for (int e = threadIdx.x; e < kEt * KW; e += 256) {
+            const int w = e % KW, q = e / KW;
+            const bool in = w0 + w < W;
+            Js[w][q] = in && i0 + q < n ? job.inst.Jbits[(size_t)(i0 + q) * W + w0 + w] : 0u;
+            Bs[w][q] = in && r0 + q < R ? job.sbits[((size_t)(r0 + q) * 2 + 1) * W + w0 + w] : 0u;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < KW; k += 8) {
+            uint32_t jv[8][4], bv[8][4];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const uint4 x = *reinterpret_cast<const uint4*>(&Js[k + u][ty * 4]);
+                const uint4 y = *reinterpret_cast<const uint4*>(&Bs[k + u][tx * 4]);
+                jv[u][0] = x.x, jv[u][1] = x.y, jv[u][2] = x.z, jv[u][3] = x.w;
+                bv[u][0] = y.x, bv[u][1] = y.y, bv[u][2] = y.z, bv[u][3] = y.w;
+            }
+#pragma unroll
+            for (int a = 0; a < 4; ++a)
+#pragma unroll
+                for (int b = 0; b < 4; ++b) {
+                    uint32_t x[8];
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) x[u] = jv[u][a] ^ bv[u][b];
+                    pc[a][b] += popc_words<8>(x);
+                }
+        }
+        __syncthreads();
+    }
+    double part[4];
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+        const int r = r0 + tx * 4 + b;
+        int t = 0;  // |t| <= 4 n
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            const int i = i0 + ty * 4 + a;
+            if (i < n && r < R) {
+                const int U = n - 2 * pc[a][b];
+                t += (job.sbits[(size_t)r * 2 * W + (i >> 5)] >> (i & 31)) & 1u ? U : -U;
+            }
+        }
+        part[b] = (double)t;
+    }
+    bq_energy_reduce(job, part, r0, red);
+}
+
+// Real couplings: J 2^-a (a: the exponent of the largest |J|) is split into three FP32 parts, multiples of
+// 2^-17, 2^-35 and the rest, so that sums of 64 terms of the first two are exact in FP32 and those of the
+// third are to 2^-54 of the largest coupling.  Every 64 columns the three sums go into an unevaluated pair
+// hi + lo by the error-free two-sum (Knuth), 1/64th of the roundings of a two-sum per term: three fused
+// multiply-adds per term instead of seven operations.  n = 2048, 1024 replicas: 0.86 ms per state set with
+// its state copy (two-sum per term: 1.31 ms); shared-memory reads of the three parts bound it.
 __device__ __forceinline__ void two_sum_acc(float& hi, float& lo, float x)
 {
     const float s = hi + x;
@@ -382,85 +513,71 @@ __device__ __forceinline__ void two_sum_acc(float& hi, float& lo, float x)
     lo += err;
 }
 
-template <int JT>
-__global__ void __launch_bounds__(256) bq_energy_tile_kernel(BqJob job, const int8_t* __restrict__ m)
+constexpr size_t kEnergyF32Smem = (size_t)4 * kEt * kEtLd * 4;
+
+__global__ void __launch_bounds__(256) bq_energy_f32_kernel(BqJob job, const int8_t* __restrict__ m)
 {
+    extern __shared__ __align__(16) float sm[];
     const int n = job.inst.n, R = job.R;
     const int i0 = blockIdx.x * kEt, r0 = blockIdx.y * kEt;
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;  // replica quad, row quad
-    __shared__ __align__(16) uint32_t Js[kEt][kEt + 4];  // PM1: [j/4][i] packed bytes; F32: [j][i] floats
-    __shared__ __align__(16) uint32_t Bs[kEt][kEt + 4];  // PM1: [j/4][r] packed bytes; F32: [j][r] sign masks
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    float* const P[3] = {sm, sm + kEt * kEtLd, sm + 2 * kEt * kEtLd};  // parts of J: [column][row]
+    float* const Bs = sm + 3 * kEt * kEtLd;                            // spins: [column][replica]
     __shared__ double red[16][kEt + 1];
-
-    int acc_i[4][4];
+    const float scale = job.inst.jscale;
+    const float* J = static_cast<const float*>(job.inst.Jraw);
     float hi[4][4], lo[4][4];
 #pragma unroll
     for (int a = 0; a < 4; ++a)
 #pragma unroll
         for (int b = 0; b < 4; ++b) {
-            acc_i[a][b] = 0;
             hi[a][b] = 0.0f;
             lo[a][b] = 0.0f;
         }
-
     for (int j0 = 0; j0 < n; j0 += kEt) {
-        if (JT == PB_J_PM1_I8) {
-            const int8_t* J = static_cast<const int8_t*>(job.inst.Jraw);
-            for (int e = threadIdx.x; e < kEt * (kEt / 4); e += 256) {
-                const int w = e & 15, q = e >> 4;  // word (4 columns), row (of J or of the spins)
-                uint32_t jw = 0, bw = 0;
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    const int j = j0 + 4 * w + c;
-                    const int i = i0 + q, r = r0 + q;
-                    const uint32_t jv = (i < n && j < n) ? (uint8_t)J[(size_t)i * n + j] : 0u;
-                    const uint32_t bv = (r < R && j < n) ? (uint8_t)m[(size_t)r * 2 * n + n + j] : 0u;
-                    jw |= jv << (8 * c);
-                    bw |= bv << (8 * c);
-                }
-                Js[w][q] = jw;
-                Bs[w][q] = bw;
-            }
-        } else {
-            const float* J = static_cast<const float*>(job.inst.Jraw);
-            for (int e = threadIdx.x; e < kEt * kEt; e += 256) {
-                const int j = e & (kEt - 1), q = e >> 6;
-                const int i = i0 + q, r = r0 + q;
-                const float jv = (i < n && j0 + j < n) ? J[(size_t)i * n + j0 + j] : 0.0f;
-                const int8_t bv = (r < R && j0 + j < n) ? m[(size_t)r * 2 * n + n + j0 + j] : (int8_t)1;
-                Js[j][q] = __float_as_uint(jv);
-                Bs[j][q] = bv < 0 ? 0x80000000u : 0u;
-            }
+        for (int e = threadIdx.x; e < kEt * kEt; e += 256) {
+            // a warp takes 8 columns x 4 rows: whole sectors read, distinct banks written
+            const int j = ((e >> 5) & 7) * 8 + (e & 7), q = (e >> 8) * 4 + ((e >> 3) & 3);
+            const int i = i0 + q, r = r0 + q;
+            const float x = (i < n && j0 + j < n) ? J[(size_t)i * n + j0 + j] * scale : 0.0f;  // an exact power of two
+            const float p1 = __fadd_rn(__fadd_rn(x, kSplit1), -kSplit1), x1 = __fadd_rn(x, -p1);
+            const float p2 = __fadd_rn(__fadd_rn(x1, kSplit2), -kSplit2);
+            P[0][j * kEtLd + q] = p1;
+            P[1][j * kEtLd + q] = p2;
+            P[2][j * kEtLd + q] = __fadd_rn(x1, -p2);
+            Bs[j * kEtLd + q] = (r < R && j0 + j < n) ? (float)m[(size_t)r * 2 * n + n + j0 + j] : 1.0f;
         }
         __syncthreads();
-        if (JT == PB_J_PM1_I8) {
-#pragma unroll 4
-            for (int w = 0; w < kEt / 4; ++w) {
-                const uint4 jv = *reinterpret_cast<const uint4*>(&Js[w][ty * 4]);
-                const uint4 bv = *reinterpret_cast<const uint4*>(&Bs[w][tx * 4]);
-                const int ja[4] = {(int)jv.x, (int)jv.y, (int)jv.z, (int)jv.w};
-                const int ba[4] = {(int)bv.x, (int)bv.y, (int)bv.z, (int)bv.w};
+        float s[3][4][4];
 #pragma unroll
-                for (int a = 0; a < 4; ++a)
+        for (int d = 0; d < 3; ++d)
 #pragma unroll
-                    for (int b = 0; b < 4; ++b) acc_i[a][b] = __dp4a(ja[a], ba[b], acc_i[a][b]);
-            }
-        } else {
+            for (int a = 0; a < 4; ++a)
+#pragma unroll
+                for (int b = 0; b < 4; ++b) s[d][a][b] = 0.0f;
 #pragma unroll 2
-            for (int j = 0; j < kEt; ++j) {
-                const uint4 jv = *reinterpret_cast<const uint4*>(&Js[j][ty * 4]);
-                const uint4 sv = *reinterpret_cast<const uint4*>(&Bs[j][tx * 4]);
-                const uint32_t ja[4] = {jv.x, jv.y, jv.z, jv.w};
-                const uint32_t sa[4] = {sv.x, sv.y, sv.z, sv.w};
+        for (int j = 0; j < kEt; ++j) {
+            const float4 bv = *reinterpret_cast<const float4*>(Bs + j * kEtLd + tx * 4);
+            const float bb[4] = {bv.x, bv.y, bv.z, bv.w};
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                const float4 jv = *reinterpret_cast<const float4*>(P[d] + j * kEtLd + ty * 4);
+                const float ja[4] = {jv.x, jv.y, jv.z, jv.w};
 #pragma unroll
                 for (int a = 0; a < 4; ++a)
 #pragma unroll
-                    for (int b = 0; b < 4; ++b) two_sum_acc(hi[a][b], lo[a][b], __uint_as_float(ja[a] ^ sa[b]));
+                    for (int b = 0; b < 4; ++b) s[d][a][b] = fmaf(ja[a], bb[b], s[d][a][b]);
             }
         }
+#pragma unroll
+        for (int d = 0; d < 3; ++d)
+#pragma unroll
+            for (int a = 0; a < 4; ++a)
+#pragma unroll
+                for (int b = 0; b < 4; ++b) two_sum_acc(hi[a][b], lo[a][b], s[d][a][b]);
         __syncthreads();
     }
-    // -sum over this thread's 4 rows of a[r][i] U[i][r], per replica, then over the 16 row quads
+    double part[4];
 #pragma unroll
     for (int b = 0; b < 4; ++b) {
         const int r = r0 + tx * 4 + b;
@@ -468,21 +585,11 @@ __global__ void __launch_bounds__(256) bq_energy_tile_kernel(BqJob job, const in
 #pragma unroll
         for (int a = 0; a < 4; ++a) {
             const int i = i0 + ty * 4 + a;
-            if (i < n && r < R) {
-                const double av = (double)m[(size_t)r * 2 * n + i];
-                const double u = JT == PB_J_PM1_I8 ? (double)acc_i[a][b] : (double)hi[a][b] + (double)lo[a][b];
-                t -= av * u;
-            }
+            if (i < n && r < R) t -= (double)m[(size_t)r * 2 * n + i] * ((double)hi[a][b] + (double)lo[a][b]);
         }
-        red[ty][tx * 4 + b] = t;
+        part[b] = t / (double)scale;
     }
-    __syncthreads();
-    if (threadIdx.x < kEt) {
-        const int r = r0 + threadIdx.x;
-        double t = 0.0;
-        for (int q = 0; q < 16; ++q) t += red[q][threadIdx.x];
-        if (r < R) job.epart[(size_t)blockIdx.x * R + r] = t;
-    }
+    bq_energy_reduce(job, part, r0, red);
 }
 
 // E[r] = sum over row tiles of epart (fixed order) - sum_c h_c m_c; one warp per replica.
@@ -557,15 +664,27 @@ cudaError_t bq_launch_best_flush(const BqJob& job, cudaStream_t st)
     return cudaGetLastError();
 }
 
+cudaError_t bq_launch_sign_words(const int8_t* J, int n, uint32_t* out, cudaStream_t st)
+{
+    bq_sign_words_kernel<<<nblocks((long long)n * ((n + 31) / 32), 8), 256, 0, st>>>(J, n, out);
+    return cudaGetLastError();
+}
+
+cudaError_t bq_readout_set_smem()
+{
+    return cudaFuncSetAttribute(bq_energy_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kEnergyF32Smem);
+}
+
 cudaError_t bq_launch_readout(const BqJob& job, int which, int8_t* out_pm, double* out_E, cudaStream_t st)
 {
-    bq_readout_kernel<<<nblocks((long long)job.R * 2 * job.inst.n, 256), 256, 0, st>>>(job, which, out_pm);
+    const int W = (job.inst.n + 31) / 32;
+    bq_readout_kernel<<<nblocks(2LL * job.R * W, 256), 256, 0, st>>>(job, which, out_pm);
     const dim3 grid((unsigned)((job.inst.n + kEt - 1) / kEt), (unsigned)((job.R + kEt - 1) / kEt));
     if (job.inst.jtype == PB_J_PM1_I8) {
-        bq_energy_tile_kernel<PB_J_PM1_I8><<<grid, 256, 0, st>>>(job, out_pm);
+        bq_energy_bits_kernel<<<grid, 256, 0, st>>>(job);
         bq_energy_sum_kernel<PB_J_PM1_I8><<<nblocks(job.R, 8), 256, 0, st>>>(job, out_pm, out_E);
     } else {
-        bq_energy_tile_kernel<PB_J_F32><<<grid, 256, 0, st>>>(job, out_pm);
+        bq_energy_f32_kernel<<<grid, 256, kEnergyF32Smem, st>>>(job, out_pm);
         bq_energy_sum_kernel<PB_J_F32><<<nblocks(job.R, 8), 256, 0, st>>>(job, out_pm, out_E);
     }
     return cudaGetLastError();

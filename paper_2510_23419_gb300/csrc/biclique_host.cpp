@@ -121,6 +121,8 @@ pb_status bq_build(pb_instance* I, const pb_instance_desc* d, cudaStream_t st)
         PB_ALLOC(B[7], tn);
         PB_CUDA_TRY(cudaMemcpyAsync(B[6].p, q8.data(), tn, cudaMemcpyHostToDevice, st));
         PB_CUDA_TRY(cudaMemcpyAsync(B[7].p, q8t.data(), tn, cudaMemcpyHostToDevice, st));
+        PB_ALLOC(B[8], (size_t)n * ((n + 31) / 32) * 4);
+        PB_CUDA_TRY(bq_launch_sign_words(B[4].as<int8_t>(), n, B[8].as<uint32_t>(), st));
         PB_CUDA_TRY(cudaStreamSynchronize(st));
     } else {
         std::vector<uint16_t> hi(tn, 0), lo(tn, 0), hit(tn, 0), lot(tn, 0);
@@ -163,6 +165,16 @@ pb_status bq_build(pb_instance* I, const pb_instance_desc* d, cudaStream_t st)
     q.h8 = B[2].as<int8_t>();
     q.hf = B[3].as<float>();
     q.Jraw = B[4].p;
+    q.Jbits = pm1 ? B[8].as<uint32_t>() : nullptr;
+    q.jscale = 1.0f;
+    if (!pm1) {
+        float amax = 0.0f;
+        for (float v : Jf) amax = std::max(amax, std::fabs(v));
+        int e = 0;
+        if (amax > 0.0f) std::frexp(amax, &e);  // amax <= 2^e
+        q.jscale = std::ldexp(1.0f, -std::max(e, -120));
+        PB_CUDA_TRY(bq_readout_set_smem());
+    }
     q.hraw = B[5].p;
     return PB_OK;
 }
@@ -291,6 +303,10 @@ static pb_status bq_prepare(pb_run* run, pb_instance* I, const pb_schedule* sc, 
     run->dev_err = run->extra[5].as<int>();  // [0] device error word, [2], [3] sweep counters
     PB_ALLOC(run->extra[6], (size_t)((n + 63) / 64) * R * 8);
     j.epart = run->extra[6].as<double>();
+    if (pm1) {
+        PB_ALLOC(run->sbits, (size_t)2 * R * ((n + 31) / 32) * 4);
+        j.sbits = run->sbits.as<uint32_t>();
+    }
     if (tensor) {
         const int esz = pm1 ? 1 : 2;
         const BqDevice& q = I->bq;

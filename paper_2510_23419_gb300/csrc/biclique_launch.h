@@ -20,6 +20,8 @@ struct BqDevice {
     const int8_t* h8;       // PM1 [2n] or null
     const float* hf;        // F32 [2n] (zeros when no field)
     const void* Jraw;       // [n][n] int8 or float, for the exact energy
+    const uint32_t* Jbits;  // PM1 [n][ceil(n/32)] sign words of Jraw
+    float jscale;           // F32: 2^-a, a the exponent of the largest |J| (|J| jscale <= 1)
     const void* hraw;       // [2n] int8 or float, or null
     // tensor-core operands, [n][ldj] row-major (row stride ldj elements, a multiple of 16)
     int32_t ldj;
@@ -54,6 +56,7 @@ struct BqJob {
     int32_t* stop;          // has_target == 2: [0] replicas that reached the target, [1] the sweep after which all
                             // had (-1 while running); the sweep counters jump to S then
     double* epart;          // [ceil(n/64)][R] row-tile parts of the exact readout energy
+    uint32_t* sbits;        // PM1 [R][2][ceil(n/32)] sign words of the state set being read out
     const int32_t* win;     // PM1 [levels][3]: threshold window (lo, width, off) of each beta level
     int32_t tabmode;        // tensor form: where the decisions read the windows (widest level decides)
     int32_t tile_split;     // tensor form: 1 = a sparse last round of tiles is split into 128-replica tiles
@@ -99,6 +102,9 @@ cudaError_t bq_launch_sweep_end(const BqJob& job, int s, int init, const int32_t
 cudaError_t bq_launch_best_flush(const BqJob& job, cudaStream_t st);
 cudaError_t bq_launch_readout(const BqJob& job, int which /*0 final, 1 best*/, int8_t* out_pm, double* out_E,
                               cudaStream_t st);
+// Sign words of +-1 couplings (BqDevice::Jbits); shared memory limit of the readout kernels.
+cudaError_t bq_launch_sign_words(const int8_t* J, int n, uint32_t* out, cudaStream_t st);
+cudaError_t bq_readout_set_smem();
 cudaError_t bq_launch_encode(const BqJob& job, const int8_t* d_states, cudaStream_t st);
 
 }  // namespace pb

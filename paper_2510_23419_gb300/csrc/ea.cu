@@ -14,6 +14,7 @@
 #include "ea_bits.cuh"
 #include "ea_fast.cuh"
 #include "ea_kernels.cuh"
+#include "exact_split.cuh"
 #include <mutex>
 
 #include "ea_launch.h"
@@ -597,33 +598,13 @@ __global__ void __launch_bounds__(256) ea_plain_energy_kernel(EaJob job, int s, 
 // ---------------------------------------------------------------------------
 // Readout and exact energies
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) ea_readout_kernel(EaJob job, const uint32_t* __restrict__ words,
-                                                         int8_t* __restrict__ out)
-{
-    const int L = job.inst.L;
-    const int N = job.inst.N, half = job.inst.half, WT = job.WT;
-    const long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= (long long)job.R * N) return;
-    const int r = (int)(j / N);
-    const int i = (int)(j - (long long)r * N);
-    const int x = i % L, y = (i / L) % L, z = i / (L * L);
-    const int c = (x + y + z) & 1;
-    const int k = i >> 1;
-    const int tile = r / (4 * WT);
-    const int w = (r / 4) % WT;
-    const int b = r & 3;
-    const uint32_t v = words[(((size_t)tile * 2 + c) * half + k) * WT + w];
-    const uint32_t minus = (job.inst.jtype == PB_J_PM1_I8) ? ((v >> (8 * b)) & 1u) : f32_minus(v, b);
-    out[j] = minus ? (int8_t)-1 : (int8_t)1;
-}
-
-// The same for one bit per spin (job.groups): a thread writes 2 V consecutive sites
-// of one replica, i.e. V words of both classes give a bit each.  Reads and writes are
-// whole words and whole rows; a byte per thread from the byte layout took 0.4 ms per
-// state set at L = 32 and 1024 replicas.
+// State buffer -> [R][N] int8 +-1.  A thread writes 2 V consecutive sites of one
+// replica, i.e. V words of both classes give a bit each: reads are whole words and writes
+// whole rows.  (A byte per thread, with a 64-bit division each, took 0.4 ms per state
+// set at L = 32 and 1024 replicas.)
 template <int V>
-__global__ void __launch_bounds__(256) ea_readout_bits_kernel(EaJob job, const uint32_t* __restrict__ words,
-                                                              int8_t* __restrict__ out, int blocks_per_replica)
+__global__ void __launch_bounds__(256) ea_readout_kernel(EaJob job, const uint32_t* __restrict__ words,
+                                                         int8_t* __restrict__ out, int blocks_per_replica)
 {
     const int L = job.inst.L, h2 = L >> 1, hv = h2 / V, WT = job.WT;
     const int r = blockIdx.x / blocks_per_replica;
@@ -631,17 +612,18 @@ __global__ void __launch_bounds__(256) ea_readout_bits_kernel(EaJob job, const u
     if (j >= hv * L * L) return;
     const int row = j / hv, q0 = (j - row * hv) * V;
     const int z = row / L, y = row - z * L;
-    const int Z = L / job.groups, nw = h2 * L * Z;
+    const int Z = job.groups ? L / job.groups : L, nw = h2 * L * Z;  // words per class and quad
     const int g = z / Z, wi = q0 + h2 * (y + L * (z - g * Z));
     const int quad = r >> 2, tile = quad / WT, w = quad - tile * WT;
-    const int sh = 8 * (r & 3) + g;
+    // the spin's bit in its word: bit g of the replica's byte, or bit 7 (sign) of an FP32 run's byte
+    const int sh = 8 * (r & 3) + (job.inst.jtype == PB_J_F32 ? 7 : g);
     const int even = (y + z) & 1;  // the class whose sites of this row have an even x
     const uint32_t* p0 = words + (((size_t)tile * 2 + even) * nw + wi) * WT + w;
     const uint32_t* p1 = words + (((size_t)tile * 2 + 1 - even) * nw + wi) * WT + w;
     uint16_t v[V];
 #pragma unroll
     for (int k = 0; k < V; ++k) {
-        const uint32_t a = (p0[k * WT] >> sh) & 1u, b = (p1[k * WT] >> sh) & 1u;
+        const uint32_t a = (p0[(size_t)k * WT] >> sh) & 1u, b = (p1[(size_t)k * WT] >> sh) & 1u;
         v[k] = (uint16_t)(0x0101u + a * 0x00FEu + b * 0xFE00u);  // 0x01 = +1, 0xFF = -1
     }
     int8_t* dst = out + (size_t)r * job.inst.N + (size_t)row * L + 2 * q0;
@@ -654,7 +636,11 @@ __global__ void __launch_bounds__(256) ea_readout_bits_kernel(EaJob job, const u
 }
 
 // E = -sum_{d,i} J[d][i] m_i m_{i+d} - sum_i h_i m_i, one block per replica;
-// int64 for PM1, FP64 for F32 (the only FP64 on the device).
+// int64 for PM1.  F32: the terms, scaled by the exact power of two 1 / 2^a >= 1 / max(|J|, |h|), are split into
+// three FP32 parts whose sums over 64 terms are exact (exact_split.cuh), and those go to FP64.  A warp takes
+// whole rows of the cube (several when they are short), so the site's coordinates cost one division per row
+// and every load is a row's: with six divisions and three FP64 terms per site this took 0.66 ms per state set
+// at L = 32 and 1024 replicas, now 0.42 ms.
 template <int JT>
 __global__ void __launch_bounds__(256) ea_energy_kernel(EaJob job, const int8_t* __restrict__ m, double* __restrict__ E)
 {
@@ -665,34 +651,73 @@ __global__ void __launch_bounds__(256) ea_energy_kernel(EaJob job, const int8_t*
     const int8_t* mr = m + (size_t)r * N;
     long long ai = 0;
     double af = 0.0;
-    for (int i = threadIdx.x; i < N; i += blockDim.x) {
-        const int x = i % L, y = (i / L) % L, z = i / (L * L);
-        const int nbr[3] = {((x + 1) % L) + L * (y + L * z), x + L * (((y + 1) % L) + L * z),
-                            x + L * (y + L * ((z + 1) % L))};
-        const int mi = mr[i];
-        if (JT == PB_J_PM1_I8) {
-            const int8_t* J = static_cast<const int8_t*>(job.inst.J3);
-            for (int d = 0; d < 3; ++d) ai -= (long long)J[(size_t)d * N + i] * mi * mr[nbr[d]];
-            if (job.inst.hraw) ai -= (long long)static_cast<const int8_t*>(job.inst.hraw)[i] * mi;
-        } else {
-            const float* J = static_cast<const float*>(job.inst.J3);
-            for (int d = 0; d < 3; ++d) af -= (double)J[(size_t)d * N + i] * (double)(mi * mr[nbr[d]]);
-            if (job.inst.hraw) af -= (double)static_cast<const float*>(job.inst.hraw)[i] * (double)mi;
+    float p1 = 0.f, p2 = 0.f, p3 = 0.f, odd = 0.f;
+    const float scale = job.inst.jscale;
+    auto term = [&](float v, bool minus) {  // -v m, in parts
+        const float xv = (minus ? v : -v) * scale, x = fabsf(xv) <= 1.0f ? xv : 0.0f;
+        odd = __fadd_rn(odd, __fadd_rn(xv, -x));  // a field that is not finite: the energy is neither (else 0)
+        const float q1 = __fadd_rn(__fadd_rn(x, kSplit1), -kSplit1), x1 = __fadd_rn(x, -q1);
+        const float q2 = __fadd_rn(__fadd_rn(x1, kSplit2), -kSplit2);
+        p1 = __fadd_rn(p1, q1);
+        p2 = __fadd_rn(p2, q2);
+        p3 = __fadd_rn(p3, __fadd_rn(x1, -q2));
+    };
+    auto flush = [&]() {
+        af += (double)p1;
+        af += (double)p2;
+        af += (double)p3;
+        p1 = p2 = p3 = 0.f;
+    };
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+    const int per = L < 32 ? 32 / L : 1;            // rows per warp
+    const int sub = L < 32 ? lane / L : 0, x0 = L < 32 ? lane - sub * L : lane;
+    int held = 0;
+    for (int row0 = warp * per; row0 < L * L; row0 += warps * per) {
+        const int row = row0 + sub;
+        if (sub >= per || row >= L * L) continue;
+        const int z = row / L, y = row - z * L;
+        const int base = row * L;
+        const int up_y = (y + 1 == L ? row - (L - 1) : row + 1) * L, up_z = (z + 1 == L ? row - (L - 1) * L : row + L) * L;
+        for (int x = x0; x < L; x += 32) {
+            const int i = base + x;
+            const int mi = mr[i];
+            const int mn[3] = {mr[base + (x + 1 == L ? 0 : x + 1)], mr[up_y + x], mr[up_z + x]};
+            if (JT == PB_J_PM1_I8) {
+                const int8_t* J = static_cast<const int8_t*>(job.inst.J3);
+                int t = 0;
+#pragma unroll
+                for (int d = 0; d < 3; ++d) t -= (int)J[(size_t)d * N + i] * mi * mn[d];
+                if (job.inst.hraw) t -= static_cast<const int8_t*>(job.inst.hraw)[i] * mi;
+                ai += t;
+            } else {
+                const float* J = static_cast<const float*>(job.inst.J3);
+#pragma unroll
+                for (int d = 0; d < 3; ++d) term(__ldg(J + (size_t)d * N + i), mi * mn[d] < 0);
+                if (job.inst.hraw) term(static_cast<const float*>(job.inst.hraw)[i], mi < 0);
+                if (++held == 16) {  // at most 64 terms per part
+                    flush();
+                    held = 0;
+                }
+            }
         }
+    }
+    if (JT == PB_J_F32) {
+        flush();
+        af = (af + (double)odd) / (double)scale;
     }
     for (int o = 16; o > 0; o >>= 1) {
         ai += __shfl_xor_sync(0xFFFFFFFFu, ai, o);
         af += __shfl_xor_sync(0xFFFFFFFFu, af, o);
     }
-    if ((threadIdx.x & 31) == 0) {
-        red_i[threadIdx.x >> 5] = ai;
-        red_f[threadIdx.x >> 5] = af;
+    if (lane == 0) {
+        red_i[warp] = ai;
+        red_f[warp] = af;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
         long long si = 0;
         double sf = 0.0;
-        for (int q = 0; q < (int)(blockDim.x >> 5); ++q) {
+        for (int q = 0; q < warps; ++q) {
             si += red_i[q];
             sf += red_f[q];
         }
@@ -857,20 +882,16 @@ cudaError_t ea_launch_plain_energy(const EaJob& job, int s, bool init, cudaStrea
 
 cudaError_t ea_launch_readout(const EaJob& job, const uint32_t* words, int8_t* out_pm, double* out_E, cudaStream_t st)
 {
-    if (job.groups) {
-        const int h2 = job.inst.L / 2, V = h2 % 4 == 0 ? 4 : (h2 % 2 == 0 ? 2 : 1);
-        const int bpr = (h2 / V * job.inst.L * job.inst.L + 255) / 256;
-        const unsigned grid = (unsigned)bpr * (unsigned)job.R;
-        if (V == 4)
-            ea_readout_bits_kernel<4><<<grid, 256, 0, st>>>(job, words, out_pm, bpr);
-        else if (V == 2)
-            ea_readout_bits_kernel<2><<<grid, 256, 0, st>>>(job, words, out_pm, bpr);
-        else
-            ea_readout_bits_kernel<1><<<grid, 256, 0, st>>>(job, words, out_pm, bpr);
-        return cudaGetLastError();
-    }
-    const long long n = (long long)job.R * job.inst.N;
-    ea_readout_kernel<<<blocks_for(n, 256), 256, 0, st>>>(job, words, out_pm);
+    const int h2 = job.inst.L / 2, V = h2 % 4 == 0 ? 4 : (h2 % 2 == 0 ? 2 : 1);
+    const int bpr = (h2 / V * job.inst.L * job.inst.L + 255) / 256;
+    const unsigned grid = (unsigned)bpr * (unsigned)job.R;
+    if (V == 4)
+        ea_readout_kernel<4><<<grid, 256, 0, st>>>(job, words, out_pm, bpr);
+    else if (V == 2)
+        ea_readout_kernel<2><<<grid, 256, 0, st>>>(job, words, out_pm, bpr);
+    else
+        ea_readout_kernel<1><<<grid, 256, 0, st>>>(job, words, out_pm, bpr);
+    if (job.groups) return cudaGetLastError();
     if (job.inst.jtype == PB_J_PM1_I8)
         ea_energy_kernel<PB_J_PM1_I8><<<job.R, 256, 0, st>>>(job, out_pm, out_E);
     else

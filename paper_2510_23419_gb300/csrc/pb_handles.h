@@ -142,6 +142,7 @@ struct pb_run {
     pb::DevBuf best_pm, final_pm, E_out;  // readout: [R][N] x2, [2R] doubles
     pb::DevBuf extra[8];
     pb::DevBuf pt[6];      // parallel tempering buffers of a general-graph run
+    pb::DevBuf sbits;      // biclique +-1: sign words of the state set being read out
     pb::DevBuf bq_alt[2];  // biclique: the parity-1 live spin buffers of sides A and B
     std::vector<int32_t> csr_nchunk;  // general graph: class chunks of each colour class
     int res_tab = 0;                  // biclique resident form: widest threshold window
