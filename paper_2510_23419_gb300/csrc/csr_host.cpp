@@ -173,6 +173,60 @@ pb_status csr_build(pb_instance* I, int32_t N, int64_t E, const int32_t* eu, con
     I->n_colours = k;
     I->csr_cls_off = cls_off;
     I->csr_orig = orig;
+    // resident rows
+    const bool res = pm1 && !h && maxdeg >= 1 && maxdeg <= kCsrResDegree;
+    std::vector<int32_t> rpos, rcls;
+    std::vector<uint16_t> rnbr;
+    std::vector<uint32_t> rsign, rdeg;
+    std::vector<uint32_t> rlow;
+    int npad = 0, rslots = 0;
+    if (res) {
+        rpos.resize((size_t)N);
+        rcls.assign((size_t)4 * k, 0);
+        for (int c = 0; c < k; ++c) {
+            const int n0 = cls_off[(size_t)c], ncls = cls_off[(size_t)c + 1] - n0;
+            rcls[(size_t)4 * c] = npad / 4;
+            rcls[(size_t)4 * c + 1] = (ncls + 3) / 4;
+            rcls[(size_t)4 * c + 2] = ncls;
+            for (int q = 0; q < ncls; ++q) rpos[(size_t)n0 + q] = npad + q;
+            npad += (ncls + 3) / 4 * 4;
+            int lo = 0, hi = 0;  // widest lower and upper part of a row of the class, in even slot counts
+            for (int p = n0; p < n0 + ncls; ++p) {
+                int below = 0;
+                for (int32_t a = rowptr[(size_t)p]; a < rowptr[(size_t)p + 1]; ++a) below += col[(size_t)a] < n0;
+                lo = std::max(lo, below);
+                hi = std::max(hi, rowptr[(size_t)p + 1] - rowptr[(size_t)p] - below);
+            }
+            lo = (lo + 1) / 2 * 2;
+            hi = (hi + 1) / 2 * 2;
+            rcls[(size_t)4 * c + 3] = lo | ((lo + hi) << 16);
+            rslots = std::max(rslots, lo + hi);
+        }
+    }
+    const bool res_fits = res && npad <= kCsrResSpins;
+    if (res_fits) {
+        const size_t words = (size_t)npad / 4;
+        rnbr.assign((size_t)rslots * npad, (uint16_t)npad);
+        rsign.assign((size_t)rslots * words, 0);
+        rlow.assign(words * 4, 0);
+        rdeg.assign(words, 0);
+        for (int c = 0; c < k; ++c) {
+            const int n0 = cls_off[(size_t)c], n1 = cls_off[(size_t)c + 1], lo = rcls[(size_t)4 * c + 3] & 0xFFFF;
+            for (int p = n0; p < n1; ++p) {
+                const int at = rpos[(size_t)p], w = at / 4, j = at & 3;
+                int sl = 0, sh = lo;
+                for (int32_t a = rowptr[(size_t)p]; a < rowptr[(size_t)p + 1]; ++a) {
+                    const int q = col[(size_t)a];
+                    const int u = q < n0 ? sl++ : sh++;
+                    rnbr[((size_t)u * words + w) * 4 + j] = (uint16_t)rpos[(size_t)q];
+                    if (J8[(size_t)a] < 0) rsign[(size_t)u * words + w] |= 0xFFu << (8 * j);
+                }
+                for (int b = 0; b < 4; ++b)
+                    if ((sl >> b) & 1) rlow[4 * (size_t)w + b] |= 0xFFu << (8 * j);
+                rdeg[(size_t)w] |= (uint32_t)(4 * (maxdeg - (rowptr[(size_t)p + 1] - rowptr[(size_t)p]))) << (8 * j);
+            }
+        }
+    }
     DevBuf* B = I->csr_bufs;  // 0 rowptr, 1 col, 2 J, 3 h, 4 cls_off, 5 orig, 6 colour, 7 rowneg, 8 pos
     auto up = [&](DevBuf& b, const void* src, size_t bytes) -> pb_status {
         PB_ALLOC(b, bytes);
@@ -191,6 +245,14 @@ pb_status csr_build(pb_instance* I, int32_t N, int64_t E, const int32_t* eu, con
     if ((ps = up(B[8], pos.data(), pos.size() * 4)) != PB_OK) return ps;
     if (ell && (ps = up(B[9], ellv.data(), ellv.size() * 4)) != PB_OK) return ps;
     if (ell && (ps = up(B[10], ellnd.data(), ellnd.size() * 2)) != PB_OK) return ps;
+    if (res_fits) {
+        if ((ps = up(B[11], rnbr.data(), rnbr.size() * 2)) != PB_OK) return ps;
+        if ((ps = up(B[12], rsign.data(), rsign.size() * 4)) != PB_OK) return ps;
+        if ((ps = up(B[13], rlow.data(), rlow.size() * 4)) != PB_OK) return ps;
+        if ((ps = up(B[14], rdeg.data(), rdeg.size() * 4)) != PB_OK) return ps;
+        if ((ps = up(B[15], rcls.data(), rcls.size() * 4)) != PB_OK) return ps;
+        if ((ps = up(B[16], rpos.data(), rpos.size() * 4)) != PB_OK) return ps;
+    }
     PB_CUDA_TRY(cudaStreamSynchronize(st));
     CsrDevice& g = I->csr;
     g = CsrDevice{};
@@ -213,6 +275,19 @@ pb_status csr_build(pb_instance* I, int32_t N, int64_t E, const int32_t* eu, con
     g.colour = B[6].as<int32_t>();
     g.ell = ell ? B[9].as<int4>() : nullptr;
     g.ell_nd = ell ? B[10].as<uint16_t>() : nullptr;
+    if (res_fits) {
+        g.res.npad = npad;
+        g.res.regular = 1;
+        for (int32_t p = 0; p < N; ++p)
+            if (rowptr[(size_t)p + 1] - rowptr[p] != maxdeg) g.res.regular = 0;
+        g.res.edges = (int32_t)E;
+        g.res.nbr = B[11].as<uint2>();
+        g.res.sign = B[12].as<uint32_t>();
+        g.res.lowdeg = B[13].as<uint4>();
+        g.res.degoff = B[14].as<uint32_t>();
+        g.res.cls = B[15].as<int32_t>();
+        g.res.pos = B[16].as<int32_t>();
+    }
     return PB_OK;
 }
 
@@ -402,6 +477,18 @@ pb_status csr_launch(pb_run* run, cudaStream_t st)
 {
     const CsrJob& j = run->cjob;
     PB_CUDA_TRY(cudaEventRecord(run->ev_start, st));
+    // The resident form where the instance has its rows: whole anneals from the initial state without
+    // tempering, and without stopping at a target (a stopped run's final states are those of the sweep at
+    // which all of its replicas had reached it).
+    if (j.g.res.npad && !run->resumed && !j.temp && j.has_target != 2) {
+        PB_CUDA_TRY(cudaEventRecord(run->ev_k0, st));
+        PB_CUDA_TRY(csr_launch_res(j, sm_count(), st));
+        PB_CUDA_TRY(cudaEventRecord(run->ev_k1, st));
+        PB_CUDA_TRY(csr_launch_readout(j, j.spins, run->final_pm.as<int8_t>(), run->E_out.as<double>(), st));
+        PB_CUDA_TRY(csr_launch_readout(j, j.best, run->best_pm.as<int8_t>(), run->E_out.as<double>() + run->R, st));
+        PB_CUDA_TRY(cudaEventRecord(run->ev_stop, st));
+        return PB_OK;
+    }
     if (!run->resumed) PB_CUDA_TRY(csr_launch_init(j, st));
     PB_CUDA_TRY(csr_launch_energy(j, j.spins, 0, st));
     PB_CUDA_TRY(csr_launch_sweep_end(j, j.s0 - 1, run->resumed ? 2 : 1, st));

@@ -7,6 +7,22 @@
 
 namespace pb {
 
+// Rows of the resident form (csr_res.cu): +-1 instances without fields, degree <= 15,
+// at most kCsrResSpins padded positions (else npad = 0).  Every class starts on a multiple of 4
+// positions; a word is 4 consecutive positions, arrays over words hold one entry per
+// position in its bytes or 16-bit halves.
+struct CsrResDevice {
+    int32_t npad;            // padded positions (a multiple of 4); byte npad of the state stays zero
+    int32_t regular;         // every spin has the same degree
+    int32_t edges;
+    const uint2* nbr;        // [slots][npad / 4] neighbour positions (npad: unused slot), lower classes first
+    const uint32_t* sign;    // [slots][npad / 4] bytes 0xFF <=> J = -1
+    const uint4* lowdeg;     // [npad / 4] bit planes (bytes 0xFF / 0) of the degree into lower classes
+    const uint32_t* degoff;  // [npad / 4] bytes 4 (maxdeg - degree)
+    const int32_t* cls;      // [n_colours][4]: first word, words, spins, slots into lower classes | all slots << 16
+    const int32_t* pos;      // [N] position of label p
+};
+
 // Device copy of a general instance.  Spins carry labels: the classes are
 // listed one after the other, each in ascending original index, and a spin's
 // label is its position in that list, so class c is the label range
@@ -33,6 +49,7 @@ struct CsrDevice {
     // spin words are kept zero; ell_nd[p] = (J = +1 count) | degree << 8
     const int4* ell;         // [N][kCsrEllSlots / 4]
     const uint16_t* ell_nd;  // [N]
+    CsrResDevice res;        // resident form
 };
 
 // Spin words: 4 replicas per uint32, one byte each, byte = 0 <=> m = +1,
@@ -73,12 +90,19 @@ struct CsrJob {
     unsigned long long* n_accept;  // [M-1] accepted exchanges per pair
 };
 
+constexpr int kCsrResThreads = 512;
+constexpr int kCsrResSpins = 65528;  // 16-bit positions; two bytes of shared memory each
+constexpr int kCsrResDegree = 15;
 constexpr int kCsrChunk = 64;  // vertices per energy chunk
 constexpr int kCsrLanesQ = 32;  // class kernel: replica words per block
 constexpr int kCsrLanesV = 8;   // class kernel: vertex lanes per block
 constexpr int kCsrEllSlots = 8;  // padded rows for +-1 instances of degree <= 8
 constexpr int kCsrMaxVpt = 16;  // class kernel: most class spins one thread takes in a launch
 
+// Resident form: the whole anneal (states, bests, target sweeps) of a run whose instance has
+// resident rows, in one launch.
+size_t csr_res_smem(int npad);
+cudaError_t csr_launch_res(const CsrJob& job, int sms, cudaStream_t st);
 cudaError_t csr_launch_init(const CsrJob& job, cudaStream_t st);
 // Blocks (class chunks) of one class launch for a class of ncls spins: whole
 // waves of resident blocks (SMs x blocks per SM of the kernel variant), at most

@@ -236,12 +236,6 @@ struct EaBitTile {
         return (J <= 2) ? 0 : (J == 3 || J == 5) ? 256 : 512;
     }
 
-    // res |= bit when r >= T (the spin is -1)
-    static __device__ __forceinline__ void decide(uint32_t r, uint32_t T, uint32_t bit, uint32_t& res)
-    {
-        asm("{\n .reg .pred p;\n setp.ge.u32 p, %1, %2;\n @p or.b32 %0, %0, %3;\n}" : "+r"(res) : "r"(r), "r"(T), "r"(bit));
-    }
-
     // The decisions of one Philox call: 4 replicas of the site of class rank k.
     template <int J>
     __device__ __forceinline__ void call(const U4& r, uint32_t k, int s, const int8_t* h, uint32_t p0, uint32_t p1,
@@ -254,20 +248,20 @@ struct EaBitTile {
             tb = htab + (s & 1) * htab_bytes + 4 * (job.nF - 1 - (6 + hv - job.fmin));
             hm[4] += hv;
             uint32_t m[4] = {0, 0, 0, 0};
-            decide(r.x, *reinterpret_cast<const uint32_t*>(tb + (X & 0xFFu)), 1u, m[0]);
-            decide(r.y, *reinterpret_cast<const uint32_t*>(tb + __byte_perm(X, 0u, 0x4441u)), 1u, m[1]);
-            decide(r.z, *reinterpret_cast<const uint32_t*>(tb + __byte_perm(X, 0u, 0x4442u)), 1u, m[2]);
-            decide(r.w, *reinterpret_cast<const uint32_t*>(tb + (X >> 24)), 1u, m[3]);
+            or_if_ge(r.x, *reinterpret_cast<const uint32_t*>(tb + (X & 0xFFu)), 1u, m[0]);
+            or_if_ge(r.y, *reinterpret_cast<const uint32_t*>(tb + __byte_perm(X, 0u, 0x4441u)), 1u, m[1]);
+            or_if_ge(r.z, *reinterpret_cast<const uint32_t*>(tb + __byte_perm(X, 0u, 0x4442u)), 1u, m[2]);
+            or_if_ge(r.w, *reinterpret_cast<const uint32_t*>(tb + (X >> 24)), 1u, m[3]);
 #pragma unroll
             for (int b = 0; b < 4; ++b) {
                 res |= m[b] << (8 * b + J);
                 hm[b] += m[b] ? hv : 0;
             }
         } else {
-            decide(r.x, *reinterpret_cast<const uint32_t*>(tb + (X & 0xFFu)), 1u << J, res);
-            decide(r.y, *reinterpret_cast<const uint32_t*>(tb + __byte_perm(X, 0u, 0x4441u)), 0x100u << J, res);
-            decide(r.z, *reinterpret_cast<const uint32_t*>(tb + __byte_perm(X, 0u, 0x4442u)), 0x10000u << J, res);
-            decide(r.w, *reinterpret_cast<const uint32_t*>(tb + (X >> 24)), 0x1000000u << J, res);
+            or_if_ge(r.x, *reinterpret_cast<const uint32_t*>(tb + (X & 0xFFu)), 1u << J, res);
+            or_if_ge(r.y, *reinterpret_cast<const uint32_t*>(tb + __byte_perm(X, 0u, 0x4441u)), 0x100u << J, res);
+            or_if_ge(r.z, *reinterpret_cast<const uint32_t*>(tb + __byte_perm(X, 0u, 0x4442u)), 0x10000u << J, res);
+            or_if_ge(r.w, *reinterpret_cast<const uint32_t*>(tb + (X >> 24)), 0x1000000u << J, res);
         }
     }
 

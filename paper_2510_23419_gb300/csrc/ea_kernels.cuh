@@ -39,6 +39,13 @@ __device__ __forceinline__ uint32_t ea_popc6_bytes(uint32_t y)
 // Decision of one replica: new spin bit (1 <=> m = -1) is 1 unless r < T.
 __device__ __forceinline__ uint32_t decide_bit(uint32_t r, uint32_t T) { return r >= T ? 1u : 0u; }
 
+// Decision of one replica into a word of spin bits: res |= bit unless r < T, as a compare
+// and a predicated or (a select and an or otherwise).
+__device__ __forceinline__ void or_if_ge(uint32_t r, uint32_t T, uint32_t bit, uint32_t& res)
+{
+    asm("{\n .reg .pred p;\n setp.ge.u32 p, %1, %2;\n @p or.b32 %0, %0, %3;\n}" : "+r"(res) : "r"(r), "r"(T), "r"(bit));
+}
+
 // 2^x on the special-function unit, results below 2^-126 flushed to zero.
 // In the decision below a flushed e cannot change the outcome: u >= 2^-24,
 // so u + u e rounds to u < 1 for every e < 2^-126.
