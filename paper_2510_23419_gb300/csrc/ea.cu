@@ -15,7 +15,9 @@
 #include "ea_fast.cuh"
 #include "ea_kernels.cuh"
 #include "exact_split.cuh"
+
 #include <mutex>
+#include <type_traits>
 
 #include "ea_launch.h"
 
@@ -27,14 +29,17 @@ namespace {
 // Resident form
 // ---------------------------------------------------------------------------
 struct TileCtx {
-    int L, WT, h2, half, N, CW, P;
-    int t, lane, warp;
-    bool active;
-    int w, q, y, zfirst, zstep;  // thread's column (q, y, w) and its z values zfirst, zfirst+zstep, ...
-    uint32_t tq;                 // Philox counter word 2 = replica quad index
+    int L, WT, h2, half, N, CW, V;
+    int t, T, lane, warp;
+    int K, part;   // K > 1: K threads share a summation lane, taking every K-th of its sites
 };
 
-__device__ __forceinline__ TileCtx tile_ctx(const EaJob& job, int tile)
+// A column's place: summation lane v < V = 2 CW is (column cw, z parity zp).
+struct Column {
+    int w, q, y, zp;
+};
+
+__device__ __forceinline__ TileCtx tile_ctx(const EaJob& job)
 {
     TileCtx g;
     g.L = job.inst.L;
@@ -43,29 +48,30 @@ __device__ __forceinline__ TileCtx tile_ctx(const EaJob& job, int tile)
     g.half = g.h2 * g.L * g.L;
     g.N = 2 * g.half;
     g.CW = g.h2 * g.L * g.WT;
-    g.P = (2 * g.CW <= kResidentThreads) ? 2 : 1;
+    g.V = 2 * g.CW;
     g.t = threadIdx.x;
+    g.T = job.threads;
     g.lane = g.t & 31;
     g.warp = g.t >> 5;
-    const int cw = (g.P == 2) ? (g.t % g.CW) : g.t;
-    g.active = g.t < g.P * g.CW;
-    g.w = g.t % g.WT;  // == cw % WT since CW and blockDim are multiples of WT
-    g.q = (cw / g.WT) % g.h2;
-    g.y = cw / (g.WT * g.h2);
-    if (g.P == 2) {
-        g.zfirst = g.t / g.CW;
-        g.zstep = 2;
-    } else {
-        g.zfirst = 0;
-        g.zstep = 1;
-    }
-    g.tq = (uint32_t)(tile * g.WT + g.w);
+    g.K = job.split;
+    g.part = g.t / g.V;
     return g;
 }
 
-// Sum 4 per-thread values over the lanes that hold the same w, then store the
-// warp's sums in part[warp][4w + b].
-__device__ __forceinline__ void warp_partials(const TileCtx& g, float v0, float v1, float v2, float v3, float* part)
+__device__ __forceinline__ Column column_of(const TileCtx& g, int v)
+{
+    Column c;
+    const int cw = v % g.CW;
+    c.zp = v / g.CW;
+    c.w = cw % g.WT;
+    c.q = (cw / g.WT) % g.h2;
+    c.y = cw / (g.WT * g.h2);
+    return c;
+}
+
+// Sum 4 values per summation lane over the lanes of a warp that hold the same w, then
+// store the warp's sums in part[vwarp][4w + b].
+__device__ __forceinline__ void warp_partials(const TileCtx& g, int vwarp, float v0, float v1, float v2, float v3, float* part)
 {
     for (int o = g.WT; o < 32; o <<= 1) {
         v0 += __shfl_xor_sync(0xFFFFFFFFu, v0, o);
@@ -74,55 +80,34 @@ __device__ __forceinline__ void warp_partials(const TileCtx& g, float v0, float 
         v3 += __shfl_xor_sync(0xFFFFFFFFu, v3, o);
     }
     if (g.lane < g.WT) {
-        float* p = part + g.warp * 4 * g.WT + 4 * g.lane;
+        float* p = part + vwarp * 4 * g.WT + 4 * g.lane;
         p[0] = v0; p[1] = v1; p[2] = v2; p[3] = v3;
     }
 }
 
-// Merge the thread's words of both colours into a global state buffer for the
-// replicas that `flags` selects (byte b = 1: replica 4w + b of each word;
-// 0x01010101: all), with the same word partition as the half-sweeps.
-__device__ __forceinline__ void tile_store_words(const TileCtx& g, const uint32_t* sp, uint32_t* gdst, int tile,
-                                                 uint32_t flags)
-{
-    if (!g.active || flags == 0u) return;
-    const int L = g.L, WT = g.WT;
-    const int h2 = L >> 1;
-    const int half = h2 * L * L;
-#pragma unroll 1
-    for (int c = 0; c < 2; ++c) {
-        const uint32_t* src = sp + (size_t)c * half * WT;
-        uint32_t* dst = gdst + ((size_t)tile * 2 + c) * half * WT;
-        for (int z = g.zfirst; z < L; z += g.zstep) {
-            const int kw = (g.q + h2 * (g.y + L * z)) * WT + g.w;
-            if (WT == 1)
-                snapshot_word<true>(dst + kw, src[kw], flags);
-            else
-                snapshot_word<false>(dst + kw, src[kw], flags);
-        }
-    }
-}
-
-// Generic tile of real couplings: any even L <= 32 without a compile-time tile.
+// Generic tile of real couplings: any even L <= 32 without a compile-time tile.  The
+// energy is summed over V = 2 CW summation lanes as in the compile-time tiles.  With
+// fewer lanes than threads (lone small jobs), K threads share a lane: each
+// updates every K-th of its sites and leaves the class-1 terms in shared memory, where
+// the lane's first thread adds them in order of z -- the same sum.
 __device__ void ea_tile(const EaJob& job, int tile, unsigned char* smem)
 {
-    const TileCtx g = tile_ctx(job, tile);
+    const TileCtx g = tile_ctx(job);
     const int L = g.L, WT = g.WT;
-    const int h2 = L >> 1;
-    const int half = h2 * L * L;
-    const int N = 2 * half;
-    const int nrep = 4 * WT;
+    const int h2 = g.h2, half = g.half, N = g.N;
+    const int nrep = 4 * WT, vwarps = (g.V + 31) / 32;
 
     // ---- shared memory carve-up (must match ea_resident_smem) ----
     uint32_t* sp = reinterpret_cast<uint32_t*>(smem);
     float* spart = reinterpret_cast<float*>(sp + (size_t)N * WT);
     uint8_t* sflag = reinterpret_cast<uint8_t*>(spart + kResidentWarps * nrep);
+    float4* const terms = reinterpret_cast<float4*>(sflag + (nrep + 15) / 16 * 16);  // [L / 2][V], K > 1 only
 
-    const uint32_t key0 = job.key0, key1 = job.key1;
     const int t = g.t;
+    const RoundKeys rk = round_keys(job.key0, job.key1);
 
     // ---- initial state (tag 1) ----
-    for (int j = t; j < N * WT; j += kResidentThreads) {
+    for (int j = t; j < N * WT; j += blockDim.x) {
         if (job.resume) {  // resumed run: the given state, in the tile layout of final_words
             sp[j] = job.final_words[(size_t)tile * N * WT + j];
             continue;
@@ -131,74 +116,130 @@ __device__ void ea_tile(const EaJob& job, int tile, unsigned char* smem)
         const int ck = j / WT;
         const int c = ck >= half ? 1 : 0;
         const int k = ck - c * half;
-        const U4 r = philox10((uint32_t)k, 0u, (uint32_t)(tile * WT + w2), (kTagInit << 24) | (uint32_t)c, key0, key1);
+        const U4 r = philox10((uint32_t)k, 0u, (uint32_t)(tile * WT + w2), (kTagInit << 24) | (uint32_t)c, job.key0, job.key1);
         sp[j] = f32_word(r.x >> 31, r.y >> 31, r.z >> 31, r.w >> 31);
     }
 
-    // One colour class: update (decide = true) or only accumulate the energy
-    // terms (decide = false, for the initial state): -m F (class 1) and -h m
-    // (class 0) per replica.
-    auto half_sweep = [&](int c, int s, bool decide, float (&ef)[4]) {
-        if (!g.active) return;
+    // One colour class over the sites of one summation lane (K > 1: this thread's part of them):
+    // update (DECIDE) or only the energy terms of the state, -m F (class 1) and -h m (class 0).
+    const float4* const j6 = reinterpret_cast<const float4*>(job.inst.j6);
+    const bool has_h = job.inst.has_h != 0;
+    auto lane_sweep = [&](auto decide, int c, int s, float cexp, int v, const Column& col, float (&ef)[4]) {
+        constexpr bool DECIDE = decltype(decide)::value;
         const uint32_t* o = sp + (size_t)(1 - c) * half * WT;
         uint32_t* own = sp + (size_t)c * half * WT;
-        const uint32_t c3 = (kTagDecision << 24) | (uint32_t)c;
-        const float cexp = f32_cexp(job.betaf[s / job.step]);
-        for (int zp = 0; zp < (g.zstep == 1 ? 2 : 1); ++zp) {
-            const int z0 = (g.zstep == 1) ? zp : g.zfirst;
-            const int px = (c + g.y + z0) & 1;
-            const EaColumn col = ea_column(L, h2, g.q, g.y, px);
-            const int oxp = col.dxp * WT, oxm = col.dxm * WT, oyp = col.dyp * WT, oym = col.dym * WT;
-            const int sz = L * h2 * WT;
+        const int px = (c + col.y + col.zp) & 1;
+        const EaColumn nbr = ea_column(L, h2, col.q, col.y, px);
+        const int oxp = nbr.dxp * WT, oxm = nbr.dxm * WT, oyp = nbr.dyp * WT, oym = nbr.dym * WT;
+        const int sz = L * h2 * WT;
+        const PhiloxPre pre = philox_pre((uint32_t)s, (uint32_t)(tile * WT + col.w), (kTagDecision << 24) | (uint32_t)c, rk);
 #pragma unroll 2
-            for (int z = z0; z < L; z += 2) {
-                const int k = g.q + h2 * (g.y + L * z);
-                const int kw = k * WT + g.w;
-                const int ozp = (z + 1 == L) ? -(L - 1) * sz : sz;
-                const int ozm = (z == 0) ? (L - 1) * sz : -sz;
-                const uint32_t nb[6] = {o[kw + oxp], o[kw + oxm], o[kw + oyp], o[kw + oym], o[kw + ozp], o[kw + ozm]};
-                const size_t site = (size_t)c * half + k;
-                const float4 ja = __ldg(reinterpret_cast<const float4*>(job.inst.j6) + 2 * site);
-                const float4 jb = __ldg(reinterpret_cast<const float4*>(job.inst.j6) + 2 * site + 1);
-                const float jv[6] = {ja.x, ja.y, ja.z, ja.w, jb.x, jb.y};
-                const float hv = jb.z;  // the site's field rides in the coupling vector
-                uint32_t snew = 0;
-                float F[4];
+        for (int j = g.part; j < h2; j += g.K) {
+            const int z = col.zp + 2 * j;
+            const int k = col.q + h2 * (col.y + L * z);
+            const int kw = k * WT + col.w;
+            const int ozp = (z + 1 == L) ? -(L - 1) * sz : sz;
+            const int ozm = (z == 0) ? (L - 1) * sz : -sz;
+            const uint32_t nb[6] = {o[kw + oxp], o[kw + oxm], o[kw + oyp], o[kw + oym], o[kw + ozp], o[kw + ozm]};
+            const size_t site = (size_t)c * half + k;
+            const float4 ja = __ldg(j6 + 2 * site);
+            const float4 jb = __ldg(j6 + 2 * site + 1);
+            const float jv[6] = {ja.x, ja.y, ja.z, ja.w, jb.x, jb.y};
+            const float hv = jb.z;  // the site's field rides in the coupling vector
+            uint32_t snew;
+            float F[4];
 #pragma unroll
-                for (int b = 0; b < 4; ++b) F[b] = ea_field_f32(jv, hv, nb, b);
-                if (decide) {
-                    const U4 r = philox10((uint32_t)k, (uint32_t)s, g.tq, c3, key0, key1);
-                    snew = decide_f32_word(r.x, r.y, r.z, r.w, F[0], F[1], F[2], F[3], cexp);
-                    own[kw] = snew;
-                } else {
-                    snew = own[kw];
-                }
+            for (int b = 0; b < 4; ++b) F[b] = ea_field_f32(jv, hv, nb, b);
+            if constexpr (DECIDE) {
+                const U4 r = philox_c0((uint32_t)k, pre, rk);
+                snew = decide_f32_word(r.x, r.y, r.z, r.w, F[0], F[1], F[2], F[3], cexp);
+                own[kw] = snew;
+            } else {
+                snew = own[kw];
+            }
+            float e[4];
 #pragma unroll
-                for (int b = 0; b < 4; ++b) {
-                    const bool dn = f32_minus(snew, b);  // m = -1
-                    if (c == 1)
-                        ef[b] += dn ? F[b] : -F[b];           // -m F
-                    else if (job.inst.has_h)
-                        ef[b] += dn ? hv : -hv;               // -h m
-                }
+            for (int b = 0; b < 4; ++b) {
+                const float x = c == 1 ? F[b] : hv;  // -m F; -h m
+                e[b] = f32_minus(snew, b) ? x : -x;
+            }
+            if (g.K > 1) {
+                // class 0 terms (fields only) come first in a lane's sum: they take the first h2 rows
+                if (c == 1 || has_h)
+                    terms[(size_t)((c == 1 && has_h ? h2 : 0) + j) * g.V + v] = make_float4(e[0], e[1], e[2], e[3]);
+            } else if (c == 1 || has_h) {
+#pragma unroll
+                for (int b = 0; b < 4; ++b) ef[b] += e[b];
             }
         }
     };
+    constexpr int kMaxV = 2;  // summation lanes per thread
+    const int lane0 = t % g.V;
+    const Column col0 = column_of(g, lane0), col1 = column_of(g, (t + g.T) % g.V);
+    auto half_sweep = [&](auto decide, int c, int s, float cexp, float (&ef)[kMaxV][4]) {
+        if (g.K > 1) {
+            if (t < g.K * g.V) lane_sweep(decide, c, s, cexp, lane0, col0, ef[0]);
+            return;
+        }
+        if (t >= g.T) return;
+        if (t < g.V) lane_sweep(decide, c, s, cexp, t, col0, ef[0]);
+        if (t + g.T < g.V) lane_sweep(decide, c, s, cexp, t + g.T, col1, ef[1]);
+    };
+    // The lanes' sums into the warp partials (every thread calls it).
+    auto partials = [&](float (&ef)[kMaxV][4]) {
+        if (g.K > 1) {
+            __syncthreads();  // the terms of class 1
+            if (t < g.V)
+                for (int j = 0; j < (has_h ? 2 : 1) * h2; ++j) {
+                    const float4 e = terms[(size_t)j * g.V + t];
+                    ef[0][0] += e.x;
+                    ef[0][1] += e.y;
+                    ef[0][2] += e.z;
+                    ef[0][3] += e.w;
+                }
+            if (g.warp < vwarps) warp_partials(g, g.warp, ef[0][0], ef[0][1], ef[0][2], ef[0][3], spart);
+            return;
+        }
+#pragma unroll
+        for (int n = 0; n < kMaxV; ++n) {
+            const int vw = g.warp + n * (g.T / 32);
+            if (t < g.T && vw < vwarps) warp_partials(g, vw, ef[n][0], ef[n][1], ef[n][2], ef[n][3], spart);
+        }
+    };
+    // Merge the lattice into a global state buffer for the replicas that the flags of a word's quad
+    // select (byte b = 1: replica 4w + b; all = 0x01010101).
+    auto store = [&](uint32_t* gdst, bool all) {
+        // a thread's words share w: blockDim and WT are powers of two apart, rows are whole
+        const uint32_t* flags = reinterpret_cast<const uint32_t*>(sflag);
+        uint32_t* dst = gdst + (size_t)tile * N * WT;
+        if (WT == 1) {
+            const uint32_t f = all ? 0x01010101u : flags[0];
+            if (f == 0u) return;
+            if (t < N) snapshot_words<true, 1>(dst + t, blockDim.x, sp + t, blockDim.x, (N - t + blockDim.x - 1) / blockDim.x, f);
+        } else {
+            const int step = (int)blockDim.x / WT * WT;  // a multiple of WT, so that w = t % WT stays
+            if (t >= step) return;
+            const uint32_t f = all ? 0x01010101u : flags[t % WT];
+            if (f == 0u) return;
+            if (t < N * WT) snapshot_words<false, 2>(dst + t, step, sp + t, step, (N * WT - t + step - 1) / step, f);
+        }
+    };
 
-    // Thread r < nrep: energy of replica r from the warp partials (fixed order).
+    // Thread r < nrep: energy of replica r from the warp partials (fixed order; warps past the lanes hold none).
     auto energy_of = [&](int r) {
         float E = 0.0f;
-        for (int v = 0; v < kResidentWarps; ++v) E += spart[v * nrep + r];
+#pragma unroll 8
+        for (int v = 0; v < vwarps; ++v) E += spart[v * nrep + r];
         return E;
     };
 
     // ---- initial energy; the initial state is the first best state (unless resumed) ----
     __syncthreads();
     {
-        float ef[4] = {0.f, 0.f, 0.f, 0.f};
-        half_sweep(0, 0, false, ef);
-        half_sweep(1, 0, false, ef);
-        warp_partials(g, ef[0], ef[1], ef[2], ef[3], spart);
+        float ef[kMaxV][4] = {};
+        half_sweep(std::false_type{}, 0, 0, 0.0f, ef);
+        half_sweep(std::false_type{}, 1, 0, 0.0f, ef);
+        partials(ef);
     }
     __syncthreads();
     int32_t hit = -1, bsweep = -1;
@@ -211,36 +252,40 @@ __device__ void ea_tile(const EaJob& job, int tile, unsigned char* smem)
             bsweep = job.best_sweep[r];
         }
     } else {
-        tile_store_words(g, sp, job.best_words, tile, 0x01010101u);
+        store(job.best_words, true);
     }
 
     // ---- sweeps ----
     const bool stop_mode = job.has_target == 2;
     for (int s = job.s0; s < job.S; ++s) {
-        float ef[4] = {0.f, 0.f, 0.f, 0.f};
-        half_sweep(0, s, true, ef);
+        float ef[kMaxV][4] = {};
+        const float cexp = f32_cexp(job.betaf[s / job.step]);
+        half_sweep(std::true_type{}, 0, s, cexp, ef);
         __syncthreads();
-        half_sweep(1, s, true, ef);
-        warp_partials(g, ef[0], ef[1], ef[2], ef[3], spart);
+        half_sweep(std::true_type{}, 1, s, cexp, ef);
+        partials(ef);
         __syncthreads();
+        bool imp = false;
         if (t < nrep) {
             const float E = energy_of(t);
             const bool live = job.has_target != 2 || hit < 0;  // stop mode: the best is frozen at the target
-            const bool imp = live && E < bestE;
+            imp = live && E < bestE;
             if (imp) bestE = E;
             if (job.has_target && hit < 0 && E <= job.target_f) hit = s;
             if (imp) bsweep = s;
             sflag[t] = imp ? 1 : 0;
         }
-        __syncthreads();
-        const uint32_t f = reinterpret_cast<const uint32_t*>(sflag)[g.w];
-        tile_store_words(g, sp, job.best_words, tile, f);
+        if (__syncthreads_or(imp)) {
+            store(job.best_words, false);
+            __syncthreads();  // the copies are read before the next sweep's class 0 changes under them
+        }
         // stop mode: the tile ends once all its replicas (padding included) have reached the target
         if (stop_mode && __syncthreads_and(t >= nrep || hit >= 0 || tile * nrep + t >= job.R)) break;
     }
 
     // ---- results ----
-    tile_store_words(g, sp, job.final_words, tile, 0x01010101u);
+    __syncthreads();
+    store(job.final_words, true);
     if (t < nrep) {
         const int r = tile * nrep + t;
         job.E_best_f[r] = bestE;
@@ -259,7 +304,7 @@ __device__ void ea_tile(const EaJob& job, int tile, unsigned char* smem)
 // of the same batch) start at once, so that kernel's CTAs take the SMs this
 // one leaves as its list runs out.
 template <int K>
-__global__ void __launch_bounds__(K <= kEaKernelPm1Split ? kBitsThreads : kResidentThreads, 1)
+__global__ void __launch_bounds__(ea_kernel_threads(K), 1)
     ea_resident_kernel(const EaJob* __restrict__ jobs, const EaWork* __restrict__ work, int n_work, int* counter)
 {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

@@ -1,14 +1,12 @@
 // ea_fast.cuh -- compile-time-shaped resident tile of the EA p-bit update for
 // real (FP32) couplings (arXiv 2510.23419: Eqs. 2-3, update groups of Sec.
 // 1.2.2, classical annealing of Sec. 1.3.1; the +-1 tile is ea_bits.cuh) for
-// cubes whose colour-class columns exactly fill
-// half the CTA: thread (cw, zp) owns the column (q, y, w) for z = zp mod 2 of
-// both colours, i.e. the sites x = 2q + parity, fixed y, every other z, for 4
-// replicas.
-//
-// Shapes whose columns fill fewer than half the CTA (L = 24: 288 column-words,
-// 576 of the 1024 threads) leave the remaining warps without sites: they take
-// part in the barriers and add zero energy partials.
+// cubes whose colour-class columns make whole warps.  Summation lane (cw, zp)
+// is the column (q, y, w) for z = zp mod 2 of both colours, i.e. the sites x =
+// 2q + parity, fixed y, every other z, for 4 replicas: its energy terms are added
+// in order of z, then over the lanes in a fixed order, so the sum does not
+// depend on the threads.  A thread takes one lane (L = 24: 576) or the two
+// of a column (L = 32, 16, 8: 1024 lanes on 512 threads).
 //
 // Same arithmetic, random words and outputs as the generic tile; what changes
 // is only the instruction budget:
@@ -28,22 +26,24 @@ constexpr int kResidentWarps = kResidentThreads / 32;
 
 template <int L, int WT>
 struct EaFastTile {
-    static constexpr int T = kResidentThreads;
     static constexpr int h2 = L / 2;
-    static constexpr int CWN = h2 * L * WT;  // column-words: two threads (z parities) per column
-    static constexpr int TB = 2 * CWN;       // threads with sites; the others only join the barriers
-    static constexpr bool kAllBusy = TB == kResidentThreads;
+    static constexpr int CWN = h2 * L * WT;  // column-words: two summation lanes (z parities) per column
+    static constexpr int TB = 2 * CWN;       // summation lanes
+    static constexpr int T = ea_f32_threads(TB, 576);
+    static constexpr int NV = TB / T;        // lanes per thread: t and t + T, the two z parities of one column
     static constexpr int half = h2 * L * L;
     static constexpr int N = 2 * half;
-    static_assert(TB <= T && TB % 32 == 0 && L % 8 == 0, "fast tile: whole warps of column-word pairs");
+    static_assert(TB % 32 == 0 && L % 8 == 0 && TB == NV * T && (NV == 1 || CWN == T), "fast tile: whole warps of columns");
     static constexpr int SZ = L * h2 * WT;  // words between z planes of a class array
     static constexpr int CLS = half * WT;   // words of one class array
     static constexpr int NREP = 4 * WT;
-    static constexpr int NW = kResidentWarps;
+    static constexpr int NW = TB / 32;
 
     const EaJob& job;
-    int tile, t, lane, warp, w, q, y, zp, base0, oyp, oym;
-    bool busy;  // the thread owns a column-word (always, when the columns fill the CTA)
+    int tile, t, lane, warp, w, q, y, zp0, base0, oyp, oym;
+    const float4* j6;
+    bool has_h;
+    bool busy;  // the thread owns a column-word (the CTA may have more threads, for other jobs)
     uint32_t tq;
     uint32_t* sp;
     float* spart;
@@ -55,15 +55,17 @@ struct EaFastTile {
         t = threadIdx.x;
         lane = t & 31;
         warp = t >> 5;
-        busy = kAllBusy || t < TB;
+        busy = t < T;
         const int cw = t % CWN;
-        zp = t / CWN;
+        zp0 = NV == 1 ? t / CWN : 0;
         w = cw % WT;
         q = (cw / WT) % h2;
         y = cw / (WT * h2);
         sp = reinterpret_cast<uint32_t*>(smem);
         spart = reinterpret_cast<float*>(sp + N * WT);
-        sflag = reinterpret_cast<uint8_t*>(spart + NW * NREP);
+        sflag = reinterpret_cast<uint8_t*>(spart + kResidentWarps * NREP);
+        j6 = reinterpret_cast<const float4*>(job.inst.j6);
+        has_h = job.inst.has_h != 0;
         rk = round_keys(job.key0, job.key1);
         tq = (uint32_t)(tile * WT + w);
         base0 = (q + h2 * y) * WT + w;
@@ -73,39 +75,32 @@ struct EaFastTile {
 
     __device__ __forceinline__ void init_state()
     {
-        if constexpr (!kAllBusy)
-            if (!busy) return;
-        if (job.resume) {  // resumed run: the given state, in the tile layout of final_words
-#pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                const uint32_t* src = job.final_words + ((size_t)tile * 2 + c) * CLS + base0;
-                for (int z = zp; z < L; z += 2) sp[c * CLS + base0 + z * SZ] = src[z * SZ];
-            }
-            return;
-        }
-#pragma unroll
+        if (!busy) return;
+#pragma unroll 1
         for (int c = 0; c < 2; ++c)
-#pragma unroll 4
-            for (int z = zp; z < L; z += 2) {
-                const int k = q + h2 * (y + L * z);
+            for (int z = NV == 1 ? zp0 : 0; z < L; z += NV == 1 ? 2 : 1) {
+                const int k = q + h2 * (y + L * z), at = c * CLS + base0 + z * SZ;
+                if (job.resume) {  // resumed run: the given state, in the tile layout of final_words
+                    sp[at] = job.final_words[(size_t)tile * 2 * CLS + at];
+                    continue;
+                }
                 const U4 r = philox10((uint32_t)k, 0u, tq, (kTagInit << 24) | (uint32_t)c, job.key0, job.key1);
-                sp[c * CLS + base0 + z * SZ] = f32_word(r.x >> 31, r.y >> 31, r.z >> 31, r.w >> 31);
+                sp[at] = f32_word(r.x >> 31, r.y >> 31, r.z >> 31, r.w >> 31);
             }
     }
 
     // One colour class: update (DECIDE) or only accumulate the energy terms of
     // the current state: -m F over class 1 and -h m over class 0.
     template <int C, bool DECIDE>
-    __device__ __forceinline__ void half_sweep(int s, float (&ef)[4])
+    __device__ __forceinline__ void half_sweep(int s, float cexp, float (&ef)[NV][4])
     {
-        if constexpr (!kAllBusy)
-            if (!busy) return;
+        if (!busy) return;
         const uint32_t* o = sp + (1 - C) * CLS;
         uint32_t* own = sp + C * CLS;
-        const int zp = this->zp;
         const PhiloxPre pre = philox_pre((uint32_t)s, tq, (kTagDecision << 24) | (uint32_t)C, rk);
-        const float cexp = f32_cexp(job.betaf[s / job.step]);
-        {
+#pragma unroll
+        for (int n = 0; n < NV; ++n) {
+            const int zp = NV == 1 ? zp0 : n;
             const int px = (C + y + zp) & 1;
             const int oxp = (px ? ((q + 1 == h2) ? -(h2 - 1) : 1) : 0) * WT;
             const int oxm = (px ? 0 : ((q == 0) ? (h2 - 1) : -1)) * WT;
@@ -115,18 +110,30 @@ struct EaFastTile {
             const uint32_t* bym = o + base0 + oym;
             const uint32_t* bz = o + base0;
             // the wrapping sites (z = 0 for the even pass, z = L-1 for the odd pass) are
-            // peeled; the others take their z neighbours at z +- 1.  One site per
-            // iteration: two would hold two sites' couplings and spill.
-            if (zp == 0) site<C, DECIDE>(0, 1, L - 1, bxp, bxm, byp, bym, bz, own, pre, cexp, ef);
-#pragma unroll 1
+            // peeled; the others take their z neighbours at z +- 1.  Two sites per
+            // iteration overlap their Philox chains and coupling loads; the terms still
+            // enter the lane's energy in order of z.
+            if (zp == 0) site<C, DECIDE>(0, 1, L - 1, couplings<C>(0), bxp, bxm, byp, bym, bz, own, pre, cexp, ef[n]);
+#pragma unroll 2
             for (int z = 2 - zp; z < L - 1 - zp; z += 2)
-                site<C, DECIDE>(z, z + 1, z - 1, bxp, bxm, byp, bym, bz, own, pre, cexp, ef);
-            if (zp == 1) site<C, DECIDE>(L - 1, 0, L - 2, bxp, bxm, byp, bym, bz, own, pre, cexp, ef);
+                site<C, DECIDE>(z, z + 1, z - 1, couplings<C>(z), bxp, bxm, byp, bym, bz, own, pre, cexp, ef[n]);
+            if (zp == 1) site<C, DECIDE>(L - 1, 0, L - 2, couplings<C>(L - 1), bxp, bxm, byp, bym, bz, own, pre, cexp, ef[n]);
         }
     }
 
+    // six couplings and the field of the column's site at z
+    struct Couplings {
+        float4 a, b;
+    };
+    template <int C>
+    __device__ __forceinline__ Couplings couplings(int z) const
+    {
+        const float4* j = j6 + 2 * (C * half + q + h2 * (y + L * z));
+        return {__ldg(j), __ldg(j + 1)};
+    }
+
     template <int C, bool DECIDE>
-    __device__ __forceinline__ void site(int z, int zup, int zdn, const uint32_t* bxp, const uint32_t* bxm,
+    __device__ __forceinline__ void site(int z, int zup, int zdn, const Couplings& j, const uint32_t* bxp, const uint32_t* bxm,
                                          const uint32_t* byp, const uint32_t* bym, const uint32_t* bz, uint32_t* own,
                                          const PhiloxPre& pre, float cexp, float (&ef)[4])
     {
@@ -134,11 +141,8 @@ struct EaFastTile {
         const uint32_t n0 = bxp[z * SZ], n1 = bxm[z * SZ], n2 = byp[z * SZ], n3 = bym[z * SZ];
         const uint32_t n4 = bz[zup * SZ], n5 = bz[zdn * SZ];
         uint32_t snew;
-        const size_t site_i = (size_t)C * half + k;
-        const float4 ja = __ldg(reinterpret_cast<const float4*>(job.inst.j6) + 2 * site_i);
-        const float4 jb = __ldg(reinterpret_cast<const float4*>(job.inst.j6) + 2 * site_i + 1);
-        const float jv[6] = {ja.x, ja.y, ja.z, ja.w, jb.x, jb.y};
-        const float hv = jb.z;  // the site's field rides in the coupling vector
+        const float jv[6] = {j.a.x, j.a.y, j.a.z, j.a.w, j.b.x, j.b.y};
+        const float hv = j.b.z;  // the site's field rides in the coupling vector
         const uint32_t nb[6] = {n0, n1, n2, n3, n4, n5};
         float F[4];
 #pragma unroll
@@ -155,27 +159,31 @@ struct EaFastTile {
             const float m = f32_sign(snew, b);  // -m F (class 1), -h m (class 0)
             if (C == 1)
                 ef[b] = fmaf(-m, F[b], ef[b]);
-            else if (job.inst.has_h)
+            else if (has_h)
                 ef[b] = fmaf(-m, hv, ef[b]);
         }
     }
 
-    __device__ __forceinline__ void partials(const float (&ef)[4])
+    __device__ __forceinline__ void partials(const float (&ef)[NV][4])
     {
-        float v0 = ef[0], v1 = ef[1], v2 = ef[2], v3 = ef[3];
+        if (warp >= T / 32) return;  // whole warps
 #pragma unroll
-        for (int o2 = WT; o2 < 32; o2 <<= 1) {
-            v0 += __shfl_xor_sync(0xFFFFFFFFu, v0, o2);
-            v1 += __shfl_xor_sync(0xFFFFFFFFu, v1, o2);
-            v2 += __shfl_xor_sync(0xFFFFFFFFu, v2, o2);
-            v3 += __shfl_xor_sync(0xFFFFFFFFu, v3, o2);
-        }
-        if (lane < WT) {
-            float* p = spart + warp * NREP + 4 * lane;
-            p[0] = v0;
-            p[1] = v1;
-            p[2] = v2;
-            p[3] = v3;
+        for (int n = 0; n < NV; ++n) {
+            float v0 = ef[n][0], v1 = ef[n][1], v2 = ef[n][2], v3 = ef[n][3];
+#pragma unroll
+            for (int o2 = WT; o2 < 32; o2 <<= 1) {
+                v0 += __shfl_xor_sync(0xFFFFFFFFu, v0, o2);
+                v1 += __shfl_xor_sync(0xFFFFFFFFu, v1, o2);
+                v2 += __shfl_xor_sync(0xFFFFFFFFu, v2, o2);
+                v3 += __shfl_xor_sync(0xFFFFFFFFu, v3, o2);
+            }
+            if (lane < WT) {
+                float* p = spart + (warp + n * (T / 32)) * NREP + 4 * lane;
+                p[0] = v0;
+                p[1] = v1;
+                p[2] = v2;
+                p[3] = v3;
+            }
         }
     }
 
@@ -191,13 +199,14 @@ struct EaFastTile {
     // that `flags` selects (byte b = 1: replica 4w + b; 0x01010101: all four)
     __device__ __forceinline__ void store_words(uint32_t* gdst, uint32_t flags) const
     {
-        if (flags == 0u || (!kAllBusy && !busy)) return;
+        if (flags == 0u || !busy) return;
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
             uint32_t* dst = gdst + ((size_t)tile * 2 + c) * CLS + base0;
             const uint32_t* src = sp + c * CLS + base0;
-#pragma unroll 4
-            for (int z = zp; z < L; z += 2) snapshot_word<WT == 1>(dst + z * SZ, src[z * SZ], flags);
+            const int z0 = NV == 1 ? zp0 * SZ : 0;
+            constexpr int dz = NV == 1 ? 2 * SZ : SZ;
+            snapshot_words<WT == 1, WT == 1 ? 2 : 8>(dst + z0, dz, src + z0, dz, NV == 1 ? L / 2 : L, flags);
         }
     }
 
@@ -206,9 +215,9 @@ struct EaFastTile {
         init_state();
         __syncthreads();
         {
-            float ef[4] = {0.f, 0.f, 0.f, 0.f};
-            half_sweep<0, false>(0, ef);
-            half_sweep<1, false>(0, ef);
+            float ef[NV][4] = {};
+            half_sweep<0, false>(0, 0.0f, ef);
+            half_sweep<1, false>(0, 0.0f, ef);
             partials(ef);
         }
         __syncthreads();
@@ -227,10 +236,11 @@ struct EaFastTile {
 
         const bool stop_mode = job.has_target == 2;
         for (int s = job.s0; s < job.S; ++s) {
-            float ef[4] = {0.f, 0.f, 0.f, 0.f};
-            half_sweep<0, true>(s, ef);
+            float ef[NV][4] = {};
+            const float cexp = f32_cexp(job.betaf[s / job.step]);
+            half_sweep<0, true>(s, cexp, ef);
             __syncthreads();
-            half_sweep<1, true>(s, ef);
+            half_sweep<1, true>(s, cexp, ef);
             partials(ef);
             __syncthreads();
             if (t < NREP) {

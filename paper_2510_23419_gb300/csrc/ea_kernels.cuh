@@ -91,28 +91,40 @@ __device__ __forceinline__ uint32_t decide_f32_word(uint32_t r0, uint32_t r1, ui
     return 0x3F3F3F3Fu | ((g << 1) & 0x80808080u);
 }
 
-// Merge the replicas of one spin word that `flags` selects (byte b = 1: replica b)
-// into a global snapshot word: the whole word when all four are selected.
-// Otherwise, with BYTES, a byte store per selected replica: the destination is
-// never read, so the snapshot does not wait on global memory (the
-// read-modify-write did, with every warp of the tile snapshotting after the same
-// barrier).  Tiles with one replica word per column (WT = 1) take it: all lanes
-// of a warp then hold the same four replicas and take the same branch.  With
-// several words per column neighbouring lanes hold different replicas, their
-// byte stores diverge, and the read-modify-write measured faster.
-template <bool BYTES>
-__device__ __forceinline__ void snapshot_word(uint32_t* dst, uint32_t v, uint32_t flags)
+// Merge the replicas that `flags` selects (byte b = 1: replica b) of the spin words
+// v[0], v[sv], ... (n of them) into the global snapshot words dst[0], dst[sd], ...: whole words
+// when all four are selected.  Otherwise, with BYTES, a byte store per selected
+// replica: the destination is never read.  Tiles with one replica word per column (WT = 1) take it:
+// all lanes of a warp then hold the same four replicas and take the same branch.  With
+// several words per column neighbouring lanes hold different replicas, their byte stores
+// diverge, and reading the old words measured faster, U of them in flight (one
+// at a time, the L = 16 tile of 16 replicas spent a third of an early sweep here).
+template <bool BYTES, int U>
+__device__ __forceinline__ void snapshot_words(uint32_t* dst, int sd, const uint32_t* v, int sv, int n, uint32_t flags)
 {
     if (flags == 0x01010101u) {
-        *dst = v;
+#pragma unroll U
+        for (int i = 0; i < n; ++i) dst[i * sd] = v[i * sv];
     } else if constexpr (BYTES) {
-        unsigned char* d = reinterpret_cast<unsigned char*>(dst);
+#pragma unroll U
+        for (int i = 0; i < n; ++i) {
+            unsigned char* d = reinterpret_cast<unsigned char*>(dst + i * sd);
+            const uint32_t x = v[i * sv];
 #pragma unroll
-        for (int b = 0; b < 4; ++b)
-            if ((flags >> (8 * b)) & 1u) d[b] = (unsigned char)(v >> (8 * b));
+            for (int b = 0; b < 4; ++b)
+                if ((flags >> (8 * b)) & 1u) d[b] = (unsigned char)(x >> (8 * b));
+        }
     } else {
         const uint32_t mask = flags * 0xFFu;
-        *dst = (*dst & ~mask) | (v & mask);
+        for (int i0 = 0; i0 < n; i0 += U) {
+            uint32_t old[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (i0 + u < n) old[u] = dst[(i0 + u) * sd];
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (i0 + u < n) dst[(i0 + u) * sd] = (old[u] & ~mask) | (v[(i0 + u) * sv] & mask);
+        }
     }
 }
 

@@ -38,8 +38,9 @@ struct EaJob {
     int32_t groups;           // 0: state buffers in the byte layout above; else (resident +-1 runs) one bit
                               // per spin, `groups` sites per word: word ((tile*2 + c)*nw + wi)*WT + w,
                               // nw = half / groups, bit 8 b + g = replica b of the quad at class rank wi + g nw
-    int32_t split;            // resident +-1 runs: the job runs on the kernel of split words (EaKernel)
-    int32_t threads;          // resident +-1 runs: threads of the CTA that take words (EaBitsShape)
+    int32_t split;            // +-1: the job runs on the kernel of split words (EaKernel); FP32: threads per
+                              // summation lane (ea_f32_split)
+    int32_t threads;          // resident runs: threads of the CTA that take words or lanes
     double* E_out[2];         // resident +-1 runs: energies of the final and the best states [R], counted
                               // from the states by the tile itself
 };
@@ -138,6 +139,15 @@ inline EaBitsShape ea_bits_shape(const EaJob& j, bool split)
     return o;
 }
 
+inline int32_t ea_tile_path_f32(int L, int WT)
+{
+    if (L == 32 && WT == 1) return kEaPathFast32;
+    if (L == 16 && WT == 4) return kEaPathFast16;
+    if (L == 8 && WT == 16) return kEaPathFast8;
+    if (L == 24 && WT == 1) return kEaPathFast24;
+    return kEaPathGeneric;
+}
+
 inline int32_t ea_tile_path(const EaJob& j)
 {
     if (j.inst.jtype == PB_J_PM1_I8) {
@@ -147,16 +157,35 @@ inline int32_t ea_tile_path(const EaJob& j)
         const bool column = cpt < G ? true : (j.inst.has_h ? false : o.column);
         return ea_bits_path(G, cpt, column, j.inst.has_h != 0);
     }
-    if (j.inst.L == 32 && j.WT == 1) return kEaPathFast32;
-    if (j.inst.L == 16 && j.WT == 4) return kEaPathFast16;
-    if (j.inst.L == 8 && j.WT == 16) return kEaPathFast8;
-    if (j.inst.L == 24 && j.WT == 1) return kEaPathFast24;
-    return kEaPathGeneric;
+    return ea_tile_path_f32(j.inst.L, j.WT);
 }
 
-inline int ea_tile_threads(const EaJob& j)
+// FP32 tiles: `lanes` = L^2 WT summation lanes (at most 1024) on 512 threads, two per thread, or one
+// per thread where they fit the kernel's CTA (`most`: ea_kernel_threads).  With 1024 threads of 64
+// registers a thread had one site in flight; with 512 it has two.  608 replicas, N(0,1), us per sweep, 1024
+// threads against this: L = 32 31.8 / 29.3, L = 16 6.9 / 5.7, L = 20 13.9 / 11.7, L = 24 15.7 / 14.1; 9728 of L = 8
+// 8.5 / 7.6.
+__host__ __device__ constexpr int ea_f32_threads(int lanes, int most) { return lanes <= most ? lanes : 512; }
+// Threads that share a summation lane: the lanes of a lone small job leave most of the CTA idle.  The
+// fewest that give the least sites per thread, within 512 threads (us per sweep at 64 replicas, one
+// thread per lane against this: L = 6 2.50 / 1.44, L = 10 3.56 / 2.39; L = 16 6.77 / 5.57).
+inline int ea_f32_split(const EaJob& j)
 {
-    return j.inst.jtype == PB_J_PM1_I8 ? ea_bits_shape(j, j.split != 0).threads : 1024;
+    if (ea_tile_path_f32(j.inst.L, j.WT) != kEaPathGeneric) return 1;
+    const int lanes = j.inst.L * j.inst.L * j.WT, sites = j.inst.L / 2;
+    int best = 1;
+    for (int k = 2; k <= sites && k * lanes <= 512; ++k)
+        if ((sites + k - 1) / k < (sites + best - 1) / best) best = k;
+    return best;
+}
+
+// Threads of the CTA (of at most `most`) that a tile of the job keeps busy, whole warps.
+inline int ea_tile_threads(const EaJob& j, int most)
+{
+    if (j.inst.jtype == PB_J_PM1_I8) return ea_bits_shape(j, j.split != 0).threads;
+    const int lanes = j.inst.L * j.inst.L * j.WT;
+    const int t = ((j.split > 1 ? j.split * lanes : ea_f32_threads(lanes, most)) + 31) / 32 * 32;
+    return t < 128 ? 128 : t;
 }
 
 // Persistent resident kernels.  For +-1 couplings, one with a thread per spin word
@@ -167,8 +196,8 @@ inline int ea_tile_threads(const EaJob& j)
 // beside L = 16, L = 8 and the runtime-shaped generic tile.  With both the
 // L = 32 and the L = 24 tile in one kernel, the register allocation they share
 // slowed the L = 32 tile by 8%.  A batch takes the L = 24 kernel when its FP32
-// tiles include L = 24 ones and no L = 32 ones; otherwise L = 24 FP32 tiles
-// run the generic tile of the first kernel.
+// tiles include ones of 576 lanes (L = 24, or 16 replicas of L = 12) and no L = 32
+// ones; otherwise L = 24 FP32 tiles run the generic tile of the first kernel.
 enum EaKernel : int32_t {
     kEaKernelPm1 = 0,
     kEaKernelPm1Split = 1,
@@ -176,6 +205,9 @@ enum EaKernel : int32_t {
     kEaKernelF32L24 = 3,
     kEaKernels = 4
 };
+// Most threads of a kernel's CTA.  576 threads leave 96 registers each (five warps on one scheduler), 512
+// leave 128.
+constexpr int ea_kernel_threads(int kernel) { return kernel == kEaKernelF32L24 ? 576 : 512; }
 // The +-1 kernel of a launch: split words if every +-1 job of it has tiles that gain.
 inline bool ea_bits_gains_by_split(const EaJob& j) { return ea_bits_shape(j, true).lanes > 1; }
 
@@ -186,12 +218,14 @@ __host__ __device__ inline size_t ea_resident_smem(int L, int WT, int jtype, int
     const size_t N = (size_t)L * L * L;
     size_t b = N * (size_t)WT * 4;          // spins [2][half][WT]
     b += (size_t)(1024 / 32) * 4 * WT * 4;  // per-warp energy partials
-    b += (size_t)4 * WT;                    // improved flags
+    b += (size_t)(4 * WT + 15) / 16 * 16;   // improved flags
+    // energy terms of shared summation lanes (generic tile, lanes <= 256): 16 bytes per lane and site of the
+    // class (of both with fields)
+    if ((size_t)L * L * WT <= 256) b += (size_t)(has_h ? 2 : 1) * (L / 2) * L * L * WT * 16;
     return (b + 127) / 128 * 128;
 }
 
 constexpr int kResidentThreads = 1024;
-constexpr int kResidentWarpsH = kResidentThreads / 32;
 constexpr int kResidentMaxWT = 32;
 constexpr size_t kResidentSmemLimit = 227 * 1024;
 

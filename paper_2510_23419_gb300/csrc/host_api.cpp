@@ -460,11 +460,12 @@ pb_status ea_batch_setup(std::vector<pb_run*>& runs, cudaStream_t st, std::share
     std::vector<EaJob> jobs;
     std::vector<TileCost> tiles[2];
     EaGroup grp[2];
-    // FP32 kernel: the one with the L = 24 tile if the batch has L = 24 FP32 tiles and no L = 32 ones
+    // FP32 kernel: the one of 576 threads if the batch has FP32 tiles of 576 lanes and no L = 32 ones (2432
+    // replicas of L = 12: 9.8 us per sweep there, 10.7 on 512 threads)
     bool f32_l24 = false, f32_l32 = false;
     for (const pb_run* r : runs) {
         if (r->job.inst.jtype != PB_J_F32) continue;
-        f32_l24 |= ea_tile_path(r->job) == kEaPathFast24;
+        f32_l24 |= r->job.inst.jtype == PB_J_F32 && r->job.inst.L * r->job.inst.L * r->job.WT == 576;
         f32_l32 |= ea_tile_path(r->job) == kEaPathFast32;
     }
     bool split = true;
@@ -474,12 +475,12 @@ pb_status ea_batch_setup(std::vector<pb_run*>& runs, cudaStream_t st, std::share
     grp[1].kernel = f32_l24 && !f32_l32 ? kEaKernelF32L24 : kEaKernelF32;
     for (size_t q = 0; q < runs.size(); ++q) {
         EaJob& j = runs[q]->job;
-        j.split = split ? 1 : 0;
-        j.threads = ea_tile_threads(j);
-        jobs.push_back(j);
         const int t = j.inst.jtype == PB_J_F32 ? 1 : 0;
+        j.split = t == 1 ? ea_f32_split(j) : (split ? 1 : 0);
+        j.threads = ea_tile_threads(j, ea_kernel_threads(grp[t].kernel));
+        jobs.push_back(j);
         grp[t].smem = std::max(grp[t].smem, ea_resident_smem(j.inst.L, j.WT, j.inst.jtype, j.inst.has_h, j.nF));
-        grp[t].threads = std::max(grp[t].threads, ea_tile_threads(j));
+        grp[t].threads = std::max(grp[t].threads, j.threads);
         const double per = (double)j.inst.N * 4.0 * j.WT * std::max(1, j.S) * (t ? 2.0 : 1.0);
         for (int k = 0; k < j.n_tiles; ++k) tiles[t].push_back({(int)q, k, per});
         grp[t].cost += per * j.n_tiles;

@@ -171,7 +171,7 @@ extern "C" pb_status pb_anneal_ea_noalloc(int32_t L, const int8_t* J_dev, const 
     j.WT = WT;
     j.n_tiles = n_tiles;
     j.split = ea_bits_gains_by_split(j) ? 1 : 0;
-    j.threads = ea_tile_threads(j);
+    j.threads = ea_tile_threads(j, ea_kernel_threads(kEaKernelPm1));
     j.best_words = reinterpret_cast<uint32_t*>(S + o_best);
     j.final_words = reinterpret_cast<uint32_t*>(S + o_final);
     j.E_best_i = reinterpret_cast<int32_t*>(S + o_E);
@@ -195,7 +195,7 @@ extern "C" pb_status pb_anneal_ea_noalloc(int32_t L, const int8_t* J_dev, const 
     PB_CUDA_TRY(ea_resident_set_smem(kernel, smem));
     PB_CUDA_TRY(ea_launch_resident(kernel, reinterpret_cast<const EaJob*>(S + o_job),
                                    reinterpret_cast<const EaWork*>(S + o_work), n_tiles, reinterpret_cast<int*>(S + o_ctr),
-                                   smem, std::min(n_tiles, sms), ea_tile_threads(j), false, st));
+                                   smem, std::min(n_tiles, sms), j.threads, false, st));
     PB_CUDA_TRY(ea_launch_readout(j, j.final_words, final_states_dev, final_E_dev, st));
     PB_CUDA_TRY(ea_launch_readout(j, j.best_words, best_states_dev, best_E_dev, st));
     PB_CUDA_TRY(cudaMemcpyAsync(best_sweep_dev, j.best_sweep, (size_t)replicas * 4, cudaMemcpyDeviceToDevice, st));
