@@ -59,7 +59,8 @@ def profiled_traffic():
     import hashlib
     import re
     csrc = os.path.join(ROOT, "paper_2510_23419_gb300", "csrc")
-    files = [os.path.join(csrc, f) for f in ("ea.cu", "ea_fast.cuh", "ea_kernels.cuh", "ea_launch.h", "pb_common.h")]
+    files = [os.path.join(csrc, f) for f in ("ea.cu", "ea_bits.cuh", "ea_fast.cuh", "ea_kernels.cuh", "ea_launch.h",
+                                             "ea_philox.cuh", "pb_common.h")]
     try:
         h = hashlib.sha256()
         for f in files:
@@ -806,9 +807,9 @@ CASES = {
     "ea-L32-gauss-small": ("ea", 32, "gauss", 608, 50, "resident"),
     "ea-L16-pm1-small": ("ea", 16, "pm1", 2432, 50, "resident"),
     "ea-L16-gauss-small": ("ea", 16, "gauss", 2432, 50, "resident"),
-    "ea-L24-pm1-small": ("ea", 24, "pm1", 608, 50, "resident"),      # generic tile (WT = 1)
-    "ea-L12-pm1-small": ("ea", 12, "pm1", 2432, 50, "resident"),     # generic tile (WT = 4)
-    "ea-L24-gauss-small": ("ea", 24, "gauss", 608, 50, "resident"),  # generic tile, FP32
+    "ea-L24-pm1-small": ("ea", 24, "pm1", 608, 50, "resident"),
+    "ea-L12-pm1-small": ("ea", 12, "pm1", 2432, 50, "resident"),
+    "ea-L24-gauss-small": ("ea", 24, "gauss", 608, 50, "resident"),
     "bq-n4096-R4096-pm1-tensor": ("bq", 4096, "pm1", 4096, 2, "tensor"),
     "bq-n4096-R4096-gauss-tensor": ("bq", 4096, "gauss", 4096, 2, "tensor"),
     "bq-n4096-R1024-pm1-cudacore": ("bq", 4096, "pm1", 1024, 1, "cudacore"),

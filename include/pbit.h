@@ -106,11 +106,12 @@ typedef struct pb_schedule {
 /* How a run executes. */
 typedef enum pb_form {
     PB_FORM_AUTO = 0,      /* the autotuner's choice for the shape if it has one; else: EA resident where it fits,
-                              else plain; biclique resident where it fits, else tensor */
+                              else plain; biclique resident where it fits (and +-1 runs of 256 < n <= 512 without
+                              flags and with at most 32 replicas per SM), else tensor */
     PB_FORM_PLAIN = 1,     /* EA: spins in global memory, one launch per colour class and sweep */
     PB_FORM_RESIDENT = 2,  /* EA: persistent kernels, each replica block's lattice kept in shared memory;
-                              biclique (n <= 256 for +-1, n <= 128 for F32): one CTA per 32 replicas runs the
-                              whole anneal with J, J^T and both sides' spins in shared memory */
+                              biclique (n <= 256 for +-1, n <= 128 for F32): one CTA per 4 to 32 replicas runs
+                              the whole anneal with J, J^T and both sides' spins on the SM */
     PB_FORM_CUDACORE = 3,  /* biclique: CUDA-core field (FP32 FMA; exact integers for +-1) */
     PB_FORM_TENSOR = 4     /* biclique: tcgen05 tensor-core field (e4m3 for +-1, split BF16 for F32) */
 } pb_form;
@@ -182,7 +183,8 @@ int64_t pb_instance_spins(const pb_instance* inst);
  * no edge inside a class: else PB_ECOLOUR) or, when colour is NULL, of the
  * greedy colouring below; classes are updated in increasing colour order and a
  * spin's Philox counter word 0 is its rank in its class (ascending index).
- * Runs use the plain form (one launch per class and sweep).  Errors: PB_EINVAL
+ * +-1 runs without fields and with at most 15 neighbours per spin keep the state in shared memory
+ * (one launch); other runs use one launch per class and sweep.  Errors: PB_EINVAL
  * (edge out of range, self-loop, PM1 value not +-1, |h| > 64), PB_ECOLOUR. */
 typedef struct pb_graph_desc {
     int32_t N;
@@ -395,7 +397,7 @@ pb_status pb_wait(pb_run* run, int32_t timeout_ms);
 pb_status pb_query(pb_run* run);
 
 /* Results (each waits for the run).  Energies are recomputed from the returned
- * states on the device: exactly in int64 for PM1 instances, in FP64 for F32
+ * states on the device: exactly for PM1 instances, to FP64 accuracy for F32
  * instances.  Arrays have `replicas` entries; any pointer may be NULL.
  * best_sweep is -1 when the initial state was never beaten. */
 pb_status pb_energy(pb_run* run, double* final_E, double* best_E, int32_t* best_sweep);

@@ -230,8 +230,8 @@ constexpr int kResidentMaxWT = 32;
 constexpr size_t kResidentSmemLimit = 227 * 1024;
 
 // Largest power-of-two WT <= min(32, cap) such that the column-words of a
-// class fit half the CTA (h2*L*WT <= kResidentThreads/2: two threads, one per
-// z parity, per column) and the tile fits shared memory; 0 if none.
+// class give at most 1024 summation lanes (h2*L*WT <= kResidentThreads/2: two lanes,
+// one per z parity, per column) and the tile fits shared memory; 0 if none.
 int ea_resident_pick_wt(int L, int jtype, int has_h, int nF, int cap_words);
 
 // Opt the persistent kernel `kernel` (EaKernel) into `smem` bytes of dynamic
