@@ -202,6 +202,14 @@ pb_status csr_build(pb_instance* I, int32_t N, int64_t E, const int32_t* eu, con
             rcls[(size_t)4 * c + 3] = lo | ((lo + hi) << 16);
             rslots = std::max(rslots, lo + hi);
         }
+        int held = 0;  // words in a thread's energy count
+        for (int c = 0; c < k; ++c) {
+            auto most = [&](int cc) { return (rcls[(size_t)4 * cc + 1] + kCsrResThreads - 1) / kCsrResThreads; };
+            held += most(c);
+            if (c + 1 < k && held + most(c + 1) <= kCsrResWords) continue;
+            rcls[(size_t)4 * c + 3] |= kCsrResFlush;
+            held = 0;
+        }
     }
     const bool res_fits = res && npad <= kCsrResSpins;
     if (res_fits) {
@@ -211,7 +219,7 @@ pb_status csr_build(pb_instance* I, int32_t N, int64_t E, const int32_t* eu, con
         rlow.assign(words * 4, 0);
         rdeg.assign(words, 0);
         for (int c = 0; c < k; ++c) {
-            const int n0 = cls_off[(size_t)c], n1 = cls_off[(size_t)c + 1], lo = rcls[(size_t)4 * c + 3] & 0xFFFF;
+            const int n0 = cls_off[(size_t)c], n1 = cls_off[(size_t)c + 1], lo = rcls[(size_t)4 * c + 3] & 0xFF;
             for (int p = n0; p < n1; ++p) {
                 const int at = rpos[(size_t)p], w = at / 4, j = at & 3;
                 int sl = 0, sh = lo;

@@ -20,7 +20,8 @@
 // Energy: a row lists its neighbours in lower classes first.  When a spin is
 // updated those hold their values of this sweep, so its unsatisfied bonds to them are
 // final: their sum over all spins is U, and E = 2 U - (number of edges).
-// They are counted in bit planes too and leave the registers once per sweep.
+// They are counted in bit planes too and leave the registers once per sweep, or earlier where a thread's
+// words of the next class could overflow the planes (kCsrResWords).
 #include <algorithm>
 
 #include "csr_launch.h"
@@ -32,8 +33,8 @@ namespace pb {
 namespace {
 
 constexpr int kThreads = kCsrResThreads;
-static_assert(kCsrResDegree * ((kCsrResSpins / 4 + kCsrResThreads - 1) / kCsrResThreads) < 512, "energy planes");
-constexpr int kAcc = 9;  // planes of a thread's energy count: 15 per spin word, at most 32 words a thread and sweep
+constexpr int kAcc = kCsrResPlanes;  // planes of a thread's energy count
+static_assert((kCsrResSpins / 4 + kThreads - 1) / kThreads <= kCsrResWords, "energy planes hold a class");
 
 // Add the bits of two words to the planes p (a bit-sliced counter of P bits).
 template <int P>
@@ -58,7 +59,7 @@ __global__ void __launch_bounds__(kThreads, 1) csr_res_kernel(CsrJob job)
     unsigned char* const spins = sm;  // byte Npad stays zero: the neighbour of unused slots
     uint32_t* const best = reinterpret_cast<uint32_t*>(sm + g.npad + 16);
     __shared__ uint32_t s_tab[2][32];  // threshold rows reversed (offset 4 (maxdeg - deg) + 8 n), by sweep parity
-    __shared__ int32_t s_cls[256][4];  // class: first word, words, spins, slots (low | all << 16)
+    __shared__ int32_t s_cls[256][4];  // class: as CsrResDevice::cls
     __shared__ int32_t s_U[2][4 * Q];
     __shared__ uint8_t s_imp[4 * Q];
     const int t = threadIdx.x, lane = t & 31;
@@ -173,15 +174,19 @@ __global__ void __launch_bounds__(kThreads, 1) csr_res_kernel(CsrJob job)
         }
     };
     clear();
-    for (int c = 0; c < nc; ++c)
+    for (int c = 0; c < nc; ++c) {
+        const int slots = s_cls[c][3], lo = slots & 0xFF;
         for (int w = t; w < s_cls[c][1]; w += kThreads) {
             const int ww = s_cls[c][0] + w;
-            const int lo = s_cls[c][3] & 0xFFFF;
             uint32_t low[P], n[P];
             gather(ww, lo, lo, low, n);
             count(low, reinterpret_cast<uint32_t*>(spins)[ww], ww);
         }
-    flush(s_U[1]);
+        if (slots & kCsrResFlush) {
+            flush(s_U[1]);
+            clear();
+        }
+    }
     __syncthreads();
 
     // thread r < 4 Q keeps replica r's running best
@@ -214,7 +219,6 @@ __global__ void __launch_bounds__(kThreads, 1) csr_res_kernel(CsrJob job)
     int lev = 0, in_lev = 0;
     uint32_t mask = 0;  // replicas whose energy improved in the previous sweep: their old spins go to the best state
     for (int s = 0; s < S; ++s) {
-        clear();
         // level of sweep s + 1, its row fetched beside the first class
         int nlev = lev, nin = in_lev + 1;
         if (nin == job.step) {
@@ -227,7 +231,8 @@ __global__ void __launch_bounds__(kThreads, 1) csr_res_kernel(CsrJob job)
         if (s > 0) mask = improved();
         const unsigned char* row = reinterpret_cast<const unsigned char*>(s_tab[s & 1]);
         for (int c = 0; c < nc; ++c) {
-            const int w0 = s_cls[c][0], nw = s_cls[c][1], nsp = s_cls[c][2], lo = s_cls[c][3] & 0xFFFF, all = s_cls[c][3] >> 16;
+            const int w0 = s_cls[c][0], nw = s_cls[c][1], nsp = s_cls[c][2], slots = s_cls[c][3];
+            const int lo = slots & 0xFF, all = slots >> 16;
             PhiloxPre pre[Q];
 #pragma unroll
             for (int q = 0; q < Q; ++q)
@@ -273,10 +278,12 @@ __global__ void __launch_bounds__(kThreads, 1) csr_res_kernel(CsrJob job)
                 if (lo) count(p, res, ww);
             }
             if (c == 0 && fetch) s_tab[(s + 1) & 1][kThreads - 1 - t] = next;
-            if (c + 1 < nc) __syncthreads();
+            if (slots & kCsrResFlush) {
+                flush(s_U[s & 1]);
+                clear();
+            }
+            __syncthreads();
         }
-        flush(s_U[s & 1]);
-        __syncthreads();
         finish(s);
         __syncthreads();
         lev = nlev;
