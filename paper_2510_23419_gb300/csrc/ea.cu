@@ -646,11 +646,13 @@ __global__ void __launch_bounds__(256) ea_plain_energy_kernel(EaJob job, int s, 
 // State buffer -> [R][N] int8 +-1.  A thread writes 2 V consecutive sites of one
 // replica, i.e. V words of both classes give a bit each: reads are whole words and writes
 // whole rows.  (A byte per thread, with a 64-bit division each, took 0.4 ms per state
-// set at L = 32 and 1024 replicas.)
-template <int V>
+// set at L = 32 and 1024 replicas.)  The widest V that L and the output's address allow
+// (ea_readout_sites); an odd address takes V = 0: one word of both classes, byte stores.
+template <int V0>
 __global__ void __launch_bounds__(256) ea_readout_kernel(EaJob job, const uint32_t* __restrict__ words,
                                                          int8_t* __restrict__ out, int blocks_per_replica)
 {
+    constexpr int V = V0 ? V0 : 1;
     const int L = job.inst.L, h2 = L >> 1, hv = h2 / V, WT = job.WT;
     const int r = blockIdx.x / blocks_per_replica;
     const int j = (blockIdx.x - r * blocks_per_replica) * 256 + threadIdx.x;
@@ -672,12 +674,16 @@ __global__ void __launch_bounds__(256) ea_readout_kernel(EaJob job, const uint32
         v[k] = (uint16_t)(0x0101u + a * 0x00FEu + b * 0xFE00u);  // 0x01 = +1, 0xFF = -1
     }
     int8_t* dst = out + (size_t)r * job.inst.N + (size_t)row * L + 2 * q0;
-    if constexpr (V == 4)
+    if constexpr (V0 == 4) {
         *reinterpret_cast<uint2*>(dst) = make_uint2(v[0] | ((uint32_t)v[1] << 16), v[2] | ((uint32_t)v[3] << 16));
-    else if constexpr (V == 2)
+    } else if constexpr (V0 == 2) {
         *reinterpret_cast<uint32_t*>(dst) = v[0] | ((uint32_t)v[1] << 16);
-    else
+    } else if constexpr (V0 == 1) {
         *reinterpret_cast<uint16_t*>(dst) = v[0];
+    } else {
+        dst[0] = (int8_t)v[0];
+        dst[1] = (int8_t)(v[0] >> 8);
+    }
 }
 
 // E = -sum_{d,i} J[d][i] m_i m_{i+d} - sum_i h_i m_i, one block per replica;
@@ -927,15 +933,17 @@ cudaError_t ea_launch_plain_energy(const EaJob& job, int s, bool init, cudaStrea
 
 cudaError_t ea_launch_readout(const EaJob& job, const uint32_t* words, int8_t* out_pm, double* out_E, cudaStream_t st)
 {
-    const int h2 = job.inst.L / 2, V = h2 % 4 == 0 ? 4 : (h2 % 2 == 0 ? 2 : 1);
-    const int bpr = (h2 / V * job.inst.L * job.inst.L + 255) / 256;
+    const int h2 = job.inst.L / 2, V = ea_readout_sites(job.inst.L, reinterpret_cast<uintptr_t>(out_pm));
+    const int bpr = (h2 / (V ? V : 1) * job.inst.L * job.inst.L + 255) / 256;
     const unsigned grid = (unsigned)bpr * (unsigned)job.R;
     if (V == 4)
         ea_readout_kernel<4><<<grid, 256, 0, st>>>(job, words, out_pm, bpr);
     else if (V == 2)
         ea_readout_kernel<2><<<grid, 256, 0, st>>>(job, words, out_pm, bpr);
-    else
+    else if (V == 1)
         ea_readout_kernel<1><<<grid, 256, 0, st>>>(job, words, out_pm, bpr);
+    else
+        ea_readout_kernel<0><<<grid, 256, 0, st>>>(job, words, out_pm, bpr);
     if (job.groups) return cudaGetLastError();
     if (job.inst.jtype == PB_J_PM1_I8)
         ea_energy_kernel<PB_J_PM1_I8><<<job.R, 256, 0, st>>>(job, out_pm, out_E);

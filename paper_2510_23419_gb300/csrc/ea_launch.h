@@ -251,6 +251,15 @@ cudaError_t ea_launch_philox_ceiling(uint64_t seed, int sweeps, int blocks, uint
 cudaError_t ea_launch_plain_init(const EaJob& job, cudaStream_t st);
 cudaError_t ea_launch_plain_sweep(const EaJob& job, int s, cudaStream_t st);
 cudaError_t ea_launch_plain_energy(const EaJob& job, int s, bool init, cudaStream_t st);
+// Words of each class that a thread of the readout takes: it stores twice as many bytes at once, at offsets that are
+// multiples of that from the output's address, which a caller of pb_anneal_ea_noalloc is free to choose.  0: no
+// alignment, single bytes.
+inline int ea_readout_sites(int L, uintptr_t out)
+{
+    for (int v = 4; v; v /= 2)
+        if (L / 2 % v == 0 && out % (2 * v) == 0) return v;
+    return 0;
+}
 // State buffer -> [R][N] int8 +-1, and energies recomputed from those states
 // (int64 for PM1, FP64 for F32; not where job.groups is set: the resident +-1
 // tiles have written E_out themselves).
