@@ -498,12 +498,12 @@ __global__ void __launch_bounds__(256) bq_energy_bits_kernel(BqJob job)
     bq_energy_reduce(job, part, r0, red);
 }
 
-// Real couplings: J 2^-a (a: the exponent of the largest |J|) is split into three FP32 parts, multiples of
-// 2^-17, 2^-35 and the rest, so that sums of 64 terms of the first two are exact in FP32 and those of the
-// third are to 2^-54 of the largest coupling.  Every 64 columns the three sums go into an unevaluated pair
-// hi + lo by the error-free two-sum (Knuth), 1/64th of the roundings of a two-sum per term: three fused
-// multiply-adds per term instead of seven operations.  n = 2048, 1024 replicas: 0.86 ms per state set with
-// its state copy (two-sum per term: 1.31 ms); shared-memory reads of the three parts bound it.
+// Real couplings: split into two FP32 parts whose sums over 64 terms are exact (exact_split.cuh).  Every 64
+// columns the two sums go into an unevaluated pair hi + lo by the error-free two-sum (Knuth), 1/32nd of
+// the roundings of a two-sum per term: two fused multiply-adds per term instead of seven operations.  A coupling that
+// has no such split goes into the pair by a two-sum of its own; the columns of a tile that hold one (for N(0,1)
+// draws one in ten) are known to the whole CTA.  n = 2048, 1024 replicas: 0.75 ms per state set with
+// its state copy (two-sum per term: 1.31 ms); shared-memory reads bound it.
 __device__ __forceinline__ void two_sum_acc(float& hi, float& lo, float x)
 {
     const float s = hi + x;
@@ -521,10 +521,11 @@ __global__ void __launch_bounds__(256) bq_energy_f32_kernel(BqJob job, const int
     const int n = job.inst.n, R = job.R;
     const int i0 = blockIdx.x * kEt, r0 = blockIdx.y * kEt;
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    float* const P[3] = {sm, sm + kEt * kEtLd, sm + 2 * kEt * kEtLd};  // parts of J: [column][row]
+    float* const P[3] = {sm, sm + kEt * kEtLd, sm + 2 * kEt * kEtLd};  // parts of J, J not split: [column][row]
     float* const Bs = sm + 3 * kEt * kEtLd;                            // spins: [column][replica]
     __shared__ double red[16][kEt + 1];
-    const float scale = job.inst.jscale;
+    __shared__ __align__(8) uint8_t s_whole[8];  // bit per column: some row's J is not split
+    const float unit = job.inst.junit;
     const float* J = static_cast<const float*>(job.inst.Jraw);
     float hi[4][4], lo[4][4];
 #pragma unroll
@@ -534,23 +535,30 @@ __global__ void __launch_bounds__(256) bq_energy_f32_kernel(BqJob job, const int
             hi[a][b] = 0.0f;
             lo[a][b] = 0.0f;
         }
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int j0 = 0; j0 < n; j0 += kEt) {
+        bool whole = false;
         for (int e = threadIdx.x; e < kEt * kEt; e += 256) {
             // a warp takes 8 columns x 4 rows: whole sectors read, distinct banks written
-            const int j = ((e >> 5) & 7) * 8 + (e & 7), q = (e >> 8) * 4 + ((e >> 3) & 3);
+            const int j = warp * 8 + (e & 7), q = (e >> 8) * 4 + ((e >> 3) & 3);
             const int i = i0 + q, r = r0 + q;
-            const float x = (i < n && j0 + j < n) ? J[(size_t)i * n + j0 + j] * scale : 0.0f;  // an exact power of two
-            const float p1 = __fadd_rn(__fadd_rn(x, kSplit1), -kSplit1), x1 = __fadd_rn(x, -p1);
-            const float p2 = __fadd_rn(__fadd_rn(x1, kSplit2), -kSplit2);
-            P[0][j * kEtLd + q] = p1;
-            P[1][j * kEtLd + q] = p2;
-            P[2][j * kEtLd + q] = __fadd_rn(x1, -p2);
+            const float x = (i < n && j0 + j < n) ? J[(size_t)i * n + j0 + j] : 0.0f;
+            float q1, q2;
+            const bool split = split_exact(x, unit, q1, q2);
+            whole |= !split;
+            P[0][j * kEtLd + q] = split ? q1 : 0.0f;
+            P[1][j * kEtLd + q] = split ? q2 : 0.0f;
+            P[2][j * kEtLd + q] = split ? 0.0f : x;
             Bs[j * kEtLd + q] = (r < R && j0 + j < n) ? (float)m[(size_t)r * 2 * n + n + j0 + j] : 1.0f;
         }
+        uint32_t cols = __ballot_sync(0xFFFFFFFFu, whole);  // lanes 8 apart share a column
+        cols |= cols >> 16;
+        cols |= cols >> 8;
+        if (lane == 0) s_whole[warp] = (uint8_t)cols;
         __syncthreads();
-        float s[3][4][4];
+        float s[2][4][4];
 #pragma unroll
-        for (int d = 0; d < 3; ++d)
+        for (int d = 0; d < 2; ++d)
 #pragma unroll
             for (int a = 0; a < 4; ++a)
 #pragma unroll
@@ -560,7 +568,7 @@ __global__ void __launch_bounds__(256) bq_energy_f32_kernel(BqJob job, const int
             const float4 bv = *reinterpret_cast<const float4*>(Bs + j * kEtLd + tx * 4);
             const float bb[4] = {bv.x, bv.y, bv.z, bv.w};
 #pragma unroll
-            for (int d = 0; d < 3; ++d) {
+            for (int d = 0; d < 2; ++d) {
                 const float4 jv = *reinterpret_cast<const float4*>(P[d] + j * kEtLd + ty * 4);
                 const float ja[4] = {jv.x, jv.y, jv.z, jv.w};
 #pragma unroll
@@ -570,11 +578,21 @@ __global__ void __launch_bounds__(256) bq_energy_f32_kernel(BqJob job, const int
             }
         }
 #pragma unroll
-        for (int d = 0; d < 3; ++d)
+        for (int d = 0; d < 2; ++d)
 #pragma unroll
             for (int a = 0; a < 4; ++a)
 #pragma unroll
                 for (int b = 0; b < 4; ++b) two_sum_acc(hi[a][b], lo[a][b], s[d][a][b]);
+        for (unsigned long long m = *reinterpret_cast<const unsigned long long*>(s_whole); m; m &= m - 1) {
+            const int j = __ffsll((long long)m) - 1;
+            const float4 bv = *reinterpret_cast<const float4*>(Bs + j * kEtLd + tx * 4);
+            const float4 jv = *reinterpret_cast<const float4*>(P[2] + j * kEtLd + ty * 4);
+            const float bb[4] = {bv.x, bv.y, bv.z, bv.w}, ja[4] = {jv.x, jv.y, jv.z, jv.w};
+#pragma unroll
+            for (int a = 0; a < 4; ++a)
+#pragma unroll
+                for (int b = 0; b < 4; ++b) two_sum_acc(hi[a][b], lo[a][b], ja[a] * bb[b]);
+        }
         __syncthreads();
     }
     double part[4];
@@ -587,7 +605,7 @@ __global__ void __launch_bounds__(256) bq_energy_f32_kernel(BqJob job, const int
             const int i = i0 + ty * 4 + a;
             if (i < n && r < R) t -= (double)m[(size_t)r * 2 * n + i] * ((double)hi[a][b] + (double)lo[a][b]);
         }
-        part[b] = t / (double)scale;
+        part[b] = t;
     }
     bq_energy_reduce(job, part, r0, red);
 }

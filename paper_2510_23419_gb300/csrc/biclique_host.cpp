@@ -8,6 +8,7 @@
 #include <string>
 #include <vector>
 
+#include "exact_split.cuh"
 #include "pb_handles.h"
 
 namespace pb {
@@ -166,13 +167,10 @@ pb_status bq_build(pb_instance* I, const pb_instance_desc* d, cudaStream_t st)
     q.hf = B[3].as<float>();
     q.Jraw = B[4].p;
     q.Jbits = pm1 ? B[8].as<uint32_t>() : nullptr;
-    q.jscale = 1.0f;
     if (!pm1) {
         float amax = 0.0f;
         for (float v : Jf) amax = std::max(amax, std::fabs(v));
-        int e = 0;
-        if (amax > 0.0f) std::frexp(amax, &e);  // amax <= 2^e
-        q.jscale = std::ldexp(1.0f, -std::max(e, -120));
+        q.junit = split_unit(amax);
         PB_CUDA_TRY(bq_readout_set_smem());
     }
     q.hraw = B[5].p;

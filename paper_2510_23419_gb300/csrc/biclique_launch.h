@@ -21,7 +21,7 @@ struct BqDevice {
     const float* hf;        // F32 [2n] (zeros when no field)
     const void* Jraw;       // [n][n] int8 or float, for the exact energy
     const uint32_t* Jbits;  // PM1 [n][ceil(n/32)] sign words of Jraw
-    float jscale;           // F32: 2^-a, a the exponent of the largest |J| (|J| jscale <= 1)
+    float junit;            // F32: split_unit of the largest |J|
     const void* hraw;       // [2n] int8 or float, or null
     // tensor-core operands, [n][ldj] row-major (row stride ldj elements, a multiple of 16)
     int32_t ldj;

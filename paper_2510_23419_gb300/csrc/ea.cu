@@ -687,8 +687,9 @@ __global__ void __launch_bounds__(256) ea_readout_kernel(EaJob job, const uint32
 }
 
 // E = -sum_{d,i} J[d][i] m_i m_{i+d} - sum_i h_i m_i, one block per replica;
-// int64 for PM1.  F32: the terms, scaled by the exact power of two 1 / 2^a >= 1 / max(|J|, |h|), are split into
-// three FP32 parts whose sums over 64 terms are exact (exact_split.cuh), and those go to FP64.  A warp takes
+// int64 for PM1.  F32: a term's coupling is split into three FP32 parts whose sums over 64 terms are exact
+// (exact_split.cuh) and go to FP64, the third to a sum of its own, so that small terms meet the rest
+// once; a term without a split (rare) goes there whole, in FP64.  A warp takes
 // whole rows of the cube (several when they are short), so the site's coordinates cost one division per row
 // and every load is a row's: with six divisions and three FP64 terms per site this took 0.66 ms per state set
 // at L = 32 and 1024 replicas, now 0.42 ms.
@@ -696,27 +697,18 @@ template <int JT>
 __global__ void __launch_bounds__(256) ea_energy_kernel(EaJob job, const int8_t* __restrict__ m, double* __restrict__ E)
 {
     __shared__ long long red_i[8];
-    __shared__ double red_f[8];
+    __shared__ double red_f[8], red_d[8];
     const int L = job.inst.L, N = job.inst.N;
     const int r = blockIdx.x;
     const int8_t* mr = m + (size_t)r * N;
     long long ai = 0;
-    double af = 0.0;
-    float p1 = 0.f, p2 = 0.f, p3 = 0.f, odd = 0.f;
-    const float scale = job.inst.jscale;
-    auto term = [&](float v, bool minus) {  // -v m, in parts
-        const float xv = (minus ? v : -v) * scale, x = fabsf(xv) <= 1.0f ? xv : 0.0f;
-        odd = __fadd_rn(odd, __fadd_rn(xv, -x));  // a field that is not finite: the energy is neither (else 0)
-        const float q1 = __fadd_rn(__fadd_rn(x, kSplit1), -kSplit1), x1 = __fadd_rn(x, -q1);
-        const float q2 = __fadd_rn(__fadd_rn(x1, kSplit2), -kSplit2);
-        p1 = __fadd_rn(p1, q1);
-        p2 = __fadd_rn(p2, q2);
-        p3 = __fadd_rn(p3, __fadd_rn(x1, -q2));
-    };
+    double af = 0.0, ad = 0.0;  // large parts; small parts and whole terms
+    float p1 = 0.f, p2 = 0.f, p3 = 0.f;
+    const float unit = job.inst.junit;
     auto flush = [&]() {
         af += (double)p1;
         af += (double)p2;
-        af += (double)p3;
+        ad += (double)p3;
         p1 = p2 = p3 = 0.f;
     };
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
@@ -741,10 +733,27 @@ __global__ void __launch_bounds__(256) ea_energy_kernel(EaJob job, const int8_t*
                 if (job.inst.hraw) t -= static_cast<const int8_t*>(job.inst.hraw)[i] * mi;
                 ai += t;
             } else {
+                // the site's terms -v m, loaded together; one branch for those without a split
                 const float* J = static_cast<const float*>(job.inst.J3);
+                float x[4], q[4][3];
 #pragma unroll
-                for (int d = 0; d < 3; ++d) term(__ldg(J + (size_t)d * N + i), mi * mn[d] < 0);
-                if (job.inst.hraw) term(static_cast<const float*>(job.inst.hraw)[i], mi < 0);
+                for (int d = 0; d < 3; ++d) x[d] = __ldg(J + (size_t)d * N + i);
+                x[3] = job.inst.hraw ? static_cast<const float*>(job.inst.hraw)[i] : 0.0f;
+                uint32_t whole = 0;
+#pragma unroll
+                for (int d = 0; d < 4; ++d) {
+                    if ((d < 3 ? mi * mn[d < 3 ? d : 0] : mi) > 0) x[d] = -x[d];
+                    const bool split = split_exact(x[d], unit, q[d][0], q[d][1], q[d][2]);
+                    whole |= split ? 0u : 1u << d;
+                    p1 = __fadd_rn(p1, split ? q[d][0] : 0.0f);
+                    p2 = __fadd_rn(p2, split ? q[d][1] : 0.0f);
+                    p3 = __fadd_rn(p3, split ? q[d][2] : 0.0f);
+                }
+                if (whole) {
+#pragma unroll
+                    for (int d = 0; d < 4; ++d)
+                        if (whole >> d & 1u) ad += (double)x[d];  // a field that is not finite is here too
+                }
                 if (++held == 16) {  // at most 64 terms per part
                     flush();
                     held = 0;
@@ -752,27 +761,27 @@ __global__ void __launch_bounds__(256) ea_energy_kernel(EaJob job, const int8_t*
             }
         }
     }
-    if (JT == PB_J_F32) {
-        flush();
-        af = (af + (double)odd) / (double)scale;
-    }
+    if (JT == PB_J_F32) flush();
     for (int o = 16; o > 0; o >>= 1) {
         ai += __shfl_xor_sync(0xFFFFFFFFu, ai, o);
         af += __shfl_xor_sync(0xFFFFFFFFu, af, o);
+        ad += __shfl_xor_sync(0xFFFFFFFFu, ad, o);
     }
     if (lane == 0) {
         red_i[warp] = ai;
         red_f[warp] = af;
+        red_d[warp] = ad;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
         long long si = 0;
-        double sf = 0.0;
+        double sf = 0.0, sd = 0.0;
         for (int q = 0; q < warps; ++q) {
             si += red_i[q];
             sf += red_f[q];
+            sd += red_d[q];
         }
-        E[r] = (JT == PB_J_PM1_I8) ? (double)si : sf;
+        E[r] = (JT == PB_J_PM1_I8) ? (double)si : sf + sd;
     }
 }
 

@@ -14,6 +14,7 @@
 #include <thread>
 #include <vector>
 
+#include "exact_split.cuh"
 #include "pb_handles.h"
 
 namespace pb {
@@ -306,16 +307,13 @@ static pb_status ea_build(pb_instance* I, const pb_instance_desc* d, cudaStream_
     e.hf = I->hf.as<float>();
     e.J3 = I->J3.p;
     e.hraw = I->hraw.p;
-    e.jscale = 1.0f;
     if (!pm1) {
         float amax = 0.0f;
         const float* J = static_cast<const float*>(d->J);
         for (int64_t q = 0; q < 3 * N; ++q) amax = std::max(amax, std::fabs(J[q]));
         for (int64_t q = 0; d->h && q < N; ++q)
             if (std::isfinite(hf[(size_t)q])) amax = std::max(amax, std::fabs(hf[(size_t)q]));
-        int ex = 0;
-        if (amax > 0.0f) std::frexp(amax, &ex);  // amax <= 2^ex
-        e.jscale = std::ldexp(1.0f, -std::max(ex, -120));
+        e.junit = split_unit(amax);
     }
     return PB_OK;
 }

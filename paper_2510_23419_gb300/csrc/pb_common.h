@@ -95,7 +95,7 @@ struct EaDevice {
     const float* hf;        // F32 [2][half] (zeros when no field)
     const void* J3;         // original layout [3][N] (int8 or float) for the energy recompute
     const void* hraw;       // original layout [N] (int8 or float) or null
-    float jscale;           // F32: 2^-a, a the exponent of the largest |J|, |h|
+    float junit;            // F32: split_unit of the largest |J|, |h|
 };
 
 }  // namespace pb
