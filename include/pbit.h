@@ -183,8 +183,9 @@ int64_t pb_instance_spins(const pb_instance* inst);
  * no edge inside a class: else PB_ECOLOUR) or, when colour is NULL, of the
  * greedy colouring below; classes are updated in increasing colour order and a
  * spin's Philox counter word 0 is its rank in its class (ascending index).
- * +-1 runs without fields and with at most 15 neighbours per spin keep the state in shared memory
- * (one launch); other runs use one launch per class and sweep.  Errors: PB_EINVAL
+ * Under PB_FORM_AUTO, +-1 anneals without fields and with at most 15 neighbours per spin keep the
+ * state in shared memory (one launch) unless the graph is large and the replicas are few; other runs,
+ * and PB_FORM_PLAIN, use one launch per class and sweep.  Errors: PB_EINVAL
  * (edge out of range, self-loop, PM1 value not +-1, |h| > 64), PB_ECOLOUR. */
 typedef struct pb_graph_desc {
     int32_t N;
@@ -339,7 +340,7 @@ pb_status pb_find_imin(pb_instance* inst, const pb_imin_opts* opts, void* stream
  * field present, ceil(log2 replicas)), which PB_FORM_AUTO jobs of pb_anneal_ex
  * and pb_anneal_batch then use.  Synchronous. */
 typedef struct pb_tune_result {
-    int32_t form;              /* chosen pb_form */
+    int32_t form;              /* chosen pb_form (PB_FORM_AUTO: general graphs that take the shared-memory form) */
     int32_t tile_width;        /* EA resident: replica words (4 replicas each) per tile; biclique tensor
                                   form: 1 = a sparse last round of 256-replica tiles is split into
                                   128-replica tiles (shorter latency, more SM-time), 0 = whole tiles;

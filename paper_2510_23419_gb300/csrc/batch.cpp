@@ -470,7 +470,7 @@ pb_status pb_autotune(pb_instance* I, int32_t R, int32_t probe_sweeps, void* str
         for (int w = 1; w <= wmax && cand.size() < 7; w *= 2) cand.push_back({PB_FORM_RESIDENT, w});
         cand.push_back({PB_FORM_PLAIN, 0});
     } else if (I->topo == PB_TOPO_CSR) {
-        cand.push_back({PB_FORM_PLAIN, 0});
+        cand.push_back({csr_takes_resident(I, R) ? PB_FORM_AUTO : PB_FORM_PLAIN, 0});
     } else {
         // tensor form with a sparse last round of tiles split into 128-replica tiles (wt 1) or not (wt 0)
         cand.push_back({PB_FORM_TENSOR, 1});

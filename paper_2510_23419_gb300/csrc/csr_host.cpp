@@ -179,7 +179,7 @@ pb_status csr_build(pb_instance* I, int32_t N, int64_t E, const int32_t* eu, con
     std::vector<uint16_t> rnbr;
     std::vector<uint32_t> rsign, rdeg;
     std::vector<uint32_t> rlow;
-    int npad = 0, rslots = 0;
+    int npad = 0, rslots = 0, rrounds = 0, rslot_rounds = 0;
     if (res) {
         rpos.resize((size_t)N);
         rcls.assign((size_t)4 * k, 0);
@@ -204,6 +204,9 @@ pb_status csr_build(pb_instance* I, int32_t N, int64_t E, const int32_t* eu, con
         }
         int held = 0;  // words in a thread's energy count
         for (int c = 0; c < k; ++c) {
+            const int ro = (rcls[(size_t)4 * c + 1] + kCsrResThreads - 1) / kCsrResThreads;
+            rrounds += ro;
+            rslot_rounds += ro * (rcls[(size_t)4 * c + 3] >> 16);
             auto most = [&](int cc) { return (rcls[(size_t)4 * cc + 1] + kCsrResThreads - 1) / kCsrResThreads; };
             held += most(c);
             if (c + 1 < k && held + most(c + 1) <= kCsrResWords) continue;
@@ -295,6 +298,8 @@ pb_status csr_build(pb_instance* I, int32_t N, int64_t E, const int32_t* eu, con
         g.res.degoff = B[14].as<uint32_t>();
         g.res.cls = B[15].as<int32_t>();
         g.res.pos = B[16].as<int32_t>();
+        g.res.rounds = rrounds;
+        g.res.slot_rounds = rslot_rounds;
     }
     return PB_OK;
 }
@@ -415,7 +420,18 @@ pb_status csr_setup(pb_run* run, pb_instance* I, const pb_schedule* sc, int R, u
     int step = 1;
     pb_status ps = schedule_levels(sc, betas, step);
     if (ps != PB_OK) return ps;
-    return csr_prepare(run, I, betas, step, sc->n_sweeps, R, seed, opts, st);
+    ps = csr_prepare(run, I, betas, step, sc->n_sweeps, R, seed, opts, st);
+    run->csr_resident = form == PB_FORM_AUTO && run->cjob.has_target != 2 && csr_takes_resident(I, R);
+    return ps;
+}
+
+bool csr_takes_resident(const pb_instance* I, int R)
+{
+    const CsrDevice& g = I->csr;
+    if (!g.res.npad) return false;
+    const int Rw = (R + 3) / 4, sms = sm_count();
+    return csr_res_us(g.res.rounds, g.res.slot_rounds, Rw, sms) <
+           csr_launches_us(g.n_colours, g.N, 2.0 * g.res.edges / g.N, Rw);
 }
 
 // Parallel tempering: M temperatures x C chains = M C slots; slot g = k C + r
@@ -479,16 +495,16 @@ static pb_status csr_setup_pt(pb_run* run, pb_instance* I, const double* ladder,
     return PB_OK;
 }
 
-// Plain form: one launch per colour class and sweep, then the energy of the
+// Resident form, or plain form: one launch per colour class and sweep, then the energy of the
 // sweep and the running best (Sec. 1.2.2, Eq. 2, Eq. 3).
 pb_status csr_launch(pb_run* run, cudaStream_t st)
 {
     const CsrJob& j = run->cjob;
     PB_CUDA_TRY(cudaEventRecord(run->ev_start, st));
-    // The resident form where the instance has its rows: whole anneals from the initial state without
-    // tempering, and without stopping at a target (a stopped run's final states are those of the sweep at
-    // which all of its replicas had reached it).
-    if (j.g.res.npad && !run->resumed && !j.temp && j.has_target != 2) {
+    // The resident form: whole anneals from the initial state without tempering, and without stopping at a target
+    // (a stopped run's final states are those of the sweep at which all of its replicas had reached it), where the
+    // instance has its rows and csr_takes_resident says so.
+    if (run->csr_resident && !run->resumed) {
         PB_CUDA_TRY(cudaEventRecord(run->ev_k0, st));
         PB_CUDA_TRY(csr_launch_res(j, sm_count(), st));
         PB_CUDA_TRY(cudaEventRecord(run->ev_k1, st));

@@ -331,7 +331,7 @@ cudaError_t csr_launch_res(const CsrJob& job, int sms, cudaStream_t st)
 {
     const size_t smem = csr_res_smem(job.g.res.npad);
     // two quads share a word's gathers; one while its CTAs fit the SMs in one wave
-    const bool two = job.Rw > sms, reg = job.g.res.regular != 0;
+    const bool two = csr_res_quads(job.Rw, sms) == 2, reg = job.g.res.regular != 0;
     if (job.g.maxdeg <= 7)
         return two ? (reg ? launch<3, 2, true>(job, smem, st) : launch<3, 2, false>(job, smem, st))
                    : (reg ? launch<3, 1, true>(job, smem, st) : launch<3, 1, false>(job, smem, st));

@@ -145,6 +145,7 @@ struct pb_run {
     pb::DevBuf sbits;      // biclique +-1: sign words of the state set being read out
     pb::DevBuf bq_alt[2];  // biclique: the parity-1 live spin buffers of sides A and B
     std::vector<int32_t> csr_nchunk;  // general graph: class chunks of each colour class
+    bool csr_resident = false;        // general graph: the run takes the resident form
     int res_tab = 0;                  // biclique resident form: widest threshold window
     int res_groups = 0;               // biclique resident form: quads of replicas per CTA
     size_t res_smem = 0;              // biclique resident form: dynamic shared memory per CTA
@@ -195,6 +196,8 @@ pb_status csr_build(pb_instance* I, int32_t N, int64_t n_edges, const int32_t* e
 pb_status csr_setup(pb_run* run, pb_instance* I, const pb_schedule* sc, int R, uint64_t seed,
                     const pb_anneal_opts* opts, cudaStream_t st);
 pb_status csr_launch(pb_run* run, cudaStream_t st);
+// The resident form is the faster one for a whole anneal of R replicas (false where the instance has no rows for it).
+bool csr_takes_resident(const pb_instance* I, int R);
 pb_status csr_fields(pb_instance* I, const int8_t* d_states, int R, float* d_out, cudaStream_t st);
 pb_status wait_run(pb_run* run, int32_t timeout_ms);
 // Form (and EA tile width) for a job: the caller's choice, else the autotuner's
