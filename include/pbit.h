@@ -335,12 +335,14 @@ pb_status pb_find_imin(pb_instance* inst, const pb_imin_opts* opts, void* stream
  * with a sparse last round split into half-width tiles, the CUDA-core form and,
  * where it fits, the resident form.  The
  * cost of a candidate is its sweep-loop time times the SMs it keeps busy (a
- * batch fills the SMs that a small job leaves idle); the cheapest is returned
+ * batch fills the SMs that a small job leaves idle); the cheapest of those that
+ * take at most 4 times as long as the fastest is returned
  * and stored in a process-wide table keyed by (topology, L or n, coupling type,
  * field present, ceil(log2 replicas)), which PB_FORM_AUTO jobs of pb_anneal_ex
  * and pb_anneal_batch then use.  Synchronous. */
 typedef struct pb_tune_result {
-    int32_t form;              /* chosen pb_form (PB_FORM_AUTO: general graphs that take the shared-memory form) */
+    int32_t form;              /* chosen pb_form; PB_FORM_AUTO: a form that only the library chooses (general
+                                  graphs in shared memory, +-1 bicliques of 256 < n <= 512 in the resident form) */
     int32_t tile_width;        /* EA resident: replica words (4 replicas each) per tile; biclique tensor
                                   form: 1 = a sparse last round of 256-replica tiles is split into
                                   128-replica tiles (shorter latency, more SM-time), 0 = whole tiles;

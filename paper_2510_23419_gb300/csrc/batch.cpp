@@ -476,7 +476,10 @@ pb_status pb_autotune(pb_instance* I, int32_t R, int32_t probe_sweeps, void* str
         cand.push_back({PB_FORM_TENSOR, 1});
         cand.push_back({PB_FORM_TENSOR, 0});
         cand.push_back({PB_FORM_CUDACORE, 0});
-        if (bq_resident_fits(I)) cand.push_back({PB_FORM_RESIDENT, 0});
+        if (bq_resident_fits(I))
+            cand.push_back({PB_FORM_RESIDENT, 0});
+        else if (bq_resident_wide(I, R))
+            cand.push_back({kFormResidentWide, 0});
     }
     pb_schedule sc{};
     sc.kind = PB_SCHED_LINEAR;
@@ -485,8 +488,8 @@ pb_status pb_autotune(pb_instance* I, int32_t R, int32_t probe_sweeps, void* str
     sc.beta0 = 0.1;
     sc.beta1 = 3.0;
     const int sms = sm_count();
-    double best = INFINITY;
-    int bi = -1;
+    std::vector<int> busy;  // SMs a candidate keeps busy
+    double fastest = INFINITY;
     for (size_t c = 0; c < cand.size(); ++c) {
         const int form = cand[c].first, wt = cand[c].second;
         pb_anneal_opts o{form, 0, NAN};
@@ -515,7 +518,7 @@ pb_status pb_autotune(pb_instance* I, int32_t R, int32_t probe_sweeps, void* str
             if (form == PB_FORM_TENSOR) {
                 units = std::min(sms, 2 * bq_tc_clusters(I->n, run->bjob.Rpad, I->jtype == PB_J_PM1_I8 ? 0 : 1,
                                                          wt != 0));
-            } else if (form == PB_FORM_RESIDENT) {
+            } else if (form == PB_FORM_RESIDENT || form == kFormResidentWide) {
                 units = std::min(sms, ((R + 3) / 4 + run->res_groups - 1) / run->res_groups);
             } else {
                 units = std::min(sms, ((I->n + 63) / 64) * ((R + 63) / 64));
@@ -527,19 +530,34 @@ pb_status pb_autotune(pb_instance* I, int32_t R, int32_t probe_sweeps, void* str
         float ms = 0.0f;
         PB_CUDA_TRY(cudaEventElapsedTime(&ms, run->batch && run->batch->ev_k0 ? run->batch->ev_k0 : run->ev_k0,
                                          run->batch && run->batch->ev_k1 ? run->batch->ev_k1 : run->ev_k1));
-        out->candidate_form[c] = form;
+        out->candidate_form[c] = form == kFormResidentWide ? PB_FORM_AUTO : form;
         out->candidate_wt[c] = wt;
         out->probe_ms[c] = ms;
-        // cost in SM-time: a batch fills the SMs a small job leaves idle
-        const double cost = (double)ms * units;
-        if (cost < best) {
+        busy.push_back(units);
+        fastest = std::min(fastest, (double)ms);
+    }
+    // cost in SM-time: a batch fills the SMs a small job leaves idle.  But a job's sweeps are serial, so one of a much
+    // slower form outlasts the batch: candidates past 4 times the fastest are out (n = 256, 512 replicas, +-1: 36 us
+    // per sweep on four SMs against 1.4 on 128; without this line AUTO took the former once tuned).
+    double best = INFINITY, best_tensor = INFINITY;
+    int bi = -1, tensor_wt = 1;
+    for (size_t c = 0; c < cand.size(); ++c) {
+        const double cost = (double)out->probe_ms[c] * busy[c];
+        if (out->probe_ms[c] <= 4.0 * fastest && cost < best) {
             best = cost;
             bi = (int)c;
         }
+        if (cand[c].first == PB_FORM_TENSOR && out->probe_ms[c] <= 4.0 * fastest && cost < best_tensor) {
+            best_tensor = cost;
+            tensor_wt = cand[c].second;
+        }
     }
     out->n_candidates = (int32_t)cand.size();
-    out->form = cand[bi].first;
+    out->form = out->candidate_form[bi];
     out->tile_width = cand[bi].second;
+    // the form that only the library names is left to its rule: runs that it does not take (flags, more replicas of
+    // the same table entry) get the tensor form with the better of its tile choices
+    if (cand[bi].first == kFormResidentWide) out->tile_width = tensor_wt;
     std::lock_guard<std::mutex> lock(g_tune_mutex);
     g_tune[tune_key(I, R)] = TuneEntry{out->form, out->tile_width};
     return PB_OK;
