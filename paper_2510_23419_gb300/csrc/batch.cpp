@@ -86,8 +86,10 @@ double est_cost(const pb_instance* I, int R, int S, int form, double* compute = 
                                                   : (I->L % 8 == 0 ? 1.2e12 : 9e11);
         c = upd / rate;
     } else if (I->topo == PB_TOPO_CSR) {
-        c = upd * std::max(1, I->maxdeg) / 4e11;
-        lat = 3.0 * std::max(1, S) * 2e-6;
+        const CsrDevice& g = I->csr;
+        const double all = csr_seconds(g.res, g.n_colours, I->N, I->csr_degree, (R + 3) / 4, std::max(1, S), sm_count(),
+                                       form == PB_FORM_RESIDENT, &c);
+        lat = all - c;
     } else {
         const double flop = upd * 2.0 * I->n * (I->jtype == PB_J_F32 ? 2.0 : 1.0);
         if (form == PB_FORM_RESIDENT || form == kFormResidentWide) {
@@ -223,6 +225,8 @@ pb_status batch_start(int count, pb_instance* const* insts, const pb_schedule* s
                 return fail(PB_EUNSUPPORTED, "form not available for EA instances");
         } else if (I->topo == PB_TOPO_CSR) {
             if (form != PB_FORM_PLAIN) return fail(PB_EUNSUPPORTED, "general sparse instances run in the plain form");
+            // for its cost: the form that csr_setup will give the run
+            if (csr_run_resident(I, replicas[q], opts ? &opts[q] : nullptr)) form = PB_FORM_RESIDENT;
         } else if (form != PB_FORM_TENSOR && form != PB_FORM_CUDACORE && form != PB_FORM_RESIDENT && form != kFormResidentWide) {
             return fail(PB_EUNSUPPORTED, "form not available for biclique instances");
         }

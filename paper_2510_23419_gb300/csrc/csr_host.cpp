@@ -170,6 +170,7 @@ pb_status csr_build(pb_instance* I, int32_t N, int64_t E, const int32_t* eu, con
     I->has_h = h ? 1 : 0;
     I->hmax = hmax;
     I->maxdeg = maxdeg;
+    I->csr_degree = 2.0 * (double)E / N;
     I->n_colours = k;
     I->csr_cls_off = cls_off;
     I->csr_orig = orig;
@@ -179,7 +180,7 @@ pb_status csr_build(pb_instance* I, int32_t N, int64_t E, const int32_t* eu, con
     std::vector<uint16_t> rnbr;
     std::vector<uint32_t> rsign, rdeg;
     std::vector<uint32_t> rlow;
-    int npad = 0, rslots = 0, rrounds = 0, rslot_rounds = 0;
+    int npad = 0, rslots = 0, rrounds = 0, rslot_rounds = 0, rslot_words = 0;
     if (res) {
         rpos.resize((size_t)N);
         rcls.assign((size_t)4 * k, 0);
@@ -207,6 +208,7 @@ pb_status csr_build(pb_instance* I, int32_t N, int64_t E, const int32_t* eu, con
             const int ro = (rcls[(size_t)4 * c + 1] + kCsrResThreads - 1) / kCsrResThreads;
             rrounds += ro;
             rslot_rounds += ro * (rcls[(size_t)4 * c + 3] >> 16);
+            rslot_words += rcls[(size_t)4 * c + 1] * (rcls[(size_t)4 * c + 3] >> 16);
             auto most = [&](int cc) { return (rcls[(size_t)4 * cc + 1] + kCsrResThreads - 1) / kCsrResThreads; };
             held += most(c);
             if (c + 1 < k && held + most(c + 1) <= kCsrResWords) continue;
@@ -300,6 +302,7 @@ pb_status csr_build(pb_instance* I, int32_t N, int64_t E, const int32_t* eu, con
         g.res.pos = B[16].as<int32_t>();
         g.res.rounds = rrounds;
         g.res.slot_rounds = rslot_rounds;
+        g.res.slot_words = rslot_words;
     }
     return PB_OK;
 }
@@ -421,8 +424,15 @@ pb_status csr_setup(pb_run* run, pb_instance* I, const pb_schedule* sc, int R, u
     pb_status ps = schedule_levels(sc, betas, step);
     if (ps != PB_OK) return ps;
     ps = csr_prepare(run, I, betas, step, sc->n_sweeps, R, seed, opts, st);
-    run->csr_resident = form == PB_FORM_AUTO && run->cjob.has_target != 2 && csr_takes_resident(I, R);
+    run->csr_resident = csr_run_resident(I, R, opts);
     return ps;
+}
+
+bool csr_run_resident(const pb_instance* I, int R, const pb_anneal_opts* opts)
+{
+    if (opts && opts->form != PB_FORM_AUTO) return false;
+    const bool stops = opts && !std::isnan(opts->target_energy) && (opts->flags & PB_FLAG_STOP_AT_TARGET);
+    return !stops && csr_takes_resident(I, R);
 }
 
 bool csr_takes_resident(const pb_instance* I, int R)
@@ -430,8 +440,8 @@ bool csr_takes_resident(const pb_instance* I, int R)
     const CsrDevice& g = I->csr;
     if (!g.res.npad) return false;
     const int Rw = (R + 3) / 4, sms = sm_count();
-    return csr_res_us(g.res.rounds, g.res.slot_rounds, Rw, sms) <
-           csr_launches_us(g.n_colours, g.N, 2.0 * g.res.edges / g.N, Rw);
+    return csr_res_us(g.res, Rw, sms) <
+           csr_launches_us(g.n_colours, g.N, I->csr_degree, Rw);
 }
 
 // Parallel tempering: M temperatures x C chains = M C slots; slot g = k C + r

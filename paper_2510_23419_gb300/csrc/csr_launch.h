@@ -24,6 +24,7 @@ struct CsrResDevice {
     const int32_t* pos;      // [N] position of label p
     int32_t rounds;          // of a sweep: sum over the classes of ceil(words / kCsrResThreads)
     int32_t slot_rounds;     // the same, weighted with the class's slots
+    int32_t slot_words;      // sum over the classes of words x slots
 };
 
 // Device copy of a general instance.  Spins carry labels: the classes are
@@ -111,21 +112,33 @@ constexpr int kCsrMaxVpt = 16;  // class kernel: most class spins one thread tak
 
 // Which form a run takes.  A resident CTA sweeps all spins of one quad (two, once the quads outnumber the SMs) alone,
 // whatever the replicas; a class launch spreads them over the chip.  So large graphs with few replicas are
-// the launches' and the rest the resident form's.  us per sweep as fitted to both forms, timed on cubes of side 5
-// to 39 and on random circulants of 4 000 to 60 000 spins and degree 2 to 14 with 1 to 1024 replicas; resident /
+// the launches' and the rest the resident form's.  us per sweep as fitted to both forms (within 25%), timed on cubes of
+// side 5 to 39 and on random circulants of 4 000 to 60 000 spins and degree 2 to 14 with 1 to 1024 replicas; resident /
 // launches, e.g.: side 25, 4 replicas 20 / 34; side 31, 64 replicas 33 / 40; side 37, 64 replicas 52 / 45, 256
 // replicas 56 / 67; 60 000 spins of degree 8, 64 replicas 86 / 69, 512 replicas 91 / 132.  The choice it makes is
-// the faster form at all but two of the 140 points (those by 10%).
+// the faster form at all but six of the 140 points (those by at most 10%).
 inline int csr_res_quads(int Rw, int sms) { return Rw > sms ? 2 : 1; }
-inline double csr_res_us(int rounds, int slot_rounds, int Rw, int sms)
+inline double csr_res_us(const CsrResDevice& g, int Rw, int sms)
 {
     const int q = csr_res_quads(Rw, sms), waves = ((Rw + q - 1) / q + sms - 1) / sms;
-    return waves * (q == 1 ? 1.1 * rounds + 0.12 * slot_rounds : 1.9 * rounds + 0.13 * slot_rounds);
+    const double sw = g.slot_words / (double)kCsrResThreads;
+    return waves * (q == 1 ? 0.97 * g.rounds + 0.047 * g.slot_rounds + 0.094 * sw - 0.7
+                           : 1.8 * g.rounds + 0.027 * g.slot_rounds + 0.133 * sw - 1.3);
 }
 inline double csr_launches_us(int n_colours, int N, double degree, int Rw)
 {
     const int more = Rw > 16 ? 4 * Rw - 64 : 0;  // replicas past the first 64, which cost no more than one quad
     return 6.4 * n_colours + N * (3.8e-4 + 4.6e-6 * degree + (Rw == 1 ? 1.4e-4 : 0.0) + more * (1.9e-6 + 1.3e-7 * degree));
+}
+// Seconds of an anneal of S sweeps in either form; compute: the part of it that needs the whole chip's SMs (a resident
+// CTA holds one SM for the run's length, the launches' fixed cost holds none).
+inline double csr_seconds(const CsrResDevice& g, int n_colours, int N, double degree, int Rw, int S, int sms, bool resident,
+                          double* compute)
+{
+    const double us = resident ? csr_res_us(g, Rw, sms) : csr_launches_us(n_colours, N, degree, Rw);
+    const int q = csr_res_quads(Rw, sms), ctas = (Rw + q - 1) / q;
+    if (compute) *compute = 1e-6 * S * (resident ? us * (ctas < sms ? (double)ctas / sms : 1.0) : us - 6.4 * n_colours);
+    return 1e-6 * S * us;
 }
 // Resident form: the whole anneal (states, bests, target sweeps) of a run whose instance has
 // resident rows, in one launch.

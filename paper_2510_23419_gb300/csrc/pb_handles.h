@@ -86,6 +86,7 @@ struct pb_instance {
     pb::DevBuf bq_bufs[12];
     // general sparse instance
     int n_colours = 0;
+    double csr_degree = 0.0;           // mean degree
     std::vector<int32_t> csr_cls_off;  // host copy of the class offsets
     std::vector<int32_t> csr_orig;     // host copy of the original index of each label
     pb::CsrDevice csr{};
@@ -198,6 +199,8 @@ pb_status csr_setup(pb_run* run, pb_instance* I, const pb_schedule* sc, int R, u
 pb_status csr_launch(pb_run* run, cudaStream_t st);
 // The resident form is the faster one for a whole anneal of R replicas (false where the instance has no rows for it).
 bool csr_takes_resident(const pb_instance* I, int R);
+// ... and an anneal with these options (may be null) takes it.
+bool csr_run_resident(const pb_instance* I, int R, const pb_anneal_opts* opts);
 pb_status csr_fields(pb_instance* I, const int8_t* d_states, int R, float* d_out, cudaStream_t st);
 pb_status wait_run(pb_run* run, int32_t timeout_ms);
 // Form (and EA tile width) for a job: the caller's choice, else the autotuner's
