@@ -66,8 +66,9 @@ int64_t footprint_bytes(const pb_instance* I, const pb_schedule* sc, int R, cons
     int64_t nblk = (n + (tensor ? kBqTcRows : kBqTileRows) - 1) / (tensor ? kBqTcRows : kBqTileRows);
     if (tensor) nblk = 4 * ((nblk + 1) & ~1LL);
     const int64_t nF = 2 * (n + I->hmax) + 1;
+    const int64_t sbits = I->jtype == PB_J_PM1_I8 ? 2 * (int64_t)R * ((n + 31) / 32) * 4 : 0;  // readout's sign words
     return 4 * Rpad * ld * esz + 2 * nblk * Rpad * 4 + nlev * (I->jtype == PB_J_PM1_I8 ? nF : 1) * 4 + 3 * Rpad * 4 +
-           (n + 63) / 64 * R * 8 + out + 4096;
+           (n + 63) / 64 * R * 8 + sbits + out + 4096;
 }
 
 }  // namespace pb
