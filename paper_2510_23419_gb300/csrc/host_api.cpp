@@ -7,7 +7,6 @@
 #include <chrono>
 #include <cmath>
 #include <cstring>
-#include <exception>
 #include <memory>
 #include <new>
 #include <string>
@@ -15,6 +14,7 @@
 #include <vector>
 
 #include "exact_split.cuh"
+#include "host_pages.h"
 #include "pb_handles.h"
 
 namespace pb {
@@ -860,37 +860,6 @@ pb_status pb_energy(pb_run* run, double* final_E, double* best_E, int32_t* best_
     return PB_OK;
 }
 
-// Large outputs usually are fresh memory whose pages do not exist yet.  A device-to-host copy that takes
-// their first faults one by one ran at 14 GB/s, into present pages at 180 GB/s (33.5 MB: 2.4 against 0.19 ms),
-// so the pages are first written on four host threads (more did not help).  Every byte written here is
-// overwritten by the copy that follows.  From 32 MB on, where the C library's allocator maps fresh memory for
-// every request; smaller buffers are mostly reused ones, whose pages are there, and the threads would only
-// cost (8 MB: 0.06 -> 0.4 ms).
-static void fault_in(int8_t* out, int64_t bytes)
-{
-    constexpr int64_t kMin = 32 << 20, kPage = 4096;
-    if (bytes < kMin) return;
-    const int64_t pages = (bytes + kPage - 1) / kPage;
-    const int threads = (int)std::min(4u, std::max(1u, std::thread::hardware_concurrency()));
-    auto touch = [&](int64_t b, int64_t e) {
-        for (int64_t p = b; p < e; ++p) *static_cast<volatile int8_t*>(out + p * kPage) = 0;
-    };
-    std::vector<std::thread> ts;
-    ts.reserve((size_t)threads);
-    int64_t done = 0;  // ranges [0, done) have a thread of their own
-    try {
-        for (int k = 0; k + 1 < threads; ++k) {
-            const int64_t e = pages * (k + 1) / threads;
-            ts.emplace_back(touch, done, e);
-            done = e;
-        }
-    } catch (const std::exception&) {
-        // no more threads to be had: the rest is touched here
-    }
-    touch(done, pages);
-    for (std::thread& t : ts) t.join();
-}
-
 static pb_status copy_states(pb_run* run, const DevBuf& src, int8_t* out, int64_t out_bytes)
 {
     if (!run || !out) return fail(PB_EINVAL, "null argument");
@@ -898,7 +867,7 @@ static pb_status copy_states(pb_run* run, const DevBuf& src, int8_t* out, int64_
     if (out_bytes < need) return fail(PB_EINVAL, "output buffer too small");
     pb_status ps = wait_run(run, -1);
     if (ps != PB_OK) return ps;
-    fault_in(out, need);
+    populate_pages(out, (size_t)need);
     PB_CUDA_TRY(cudaMemcpy(out, src.p, (size_t)need, cudaMemcpyDeviceToHost));
     return PB_OK;
 }
