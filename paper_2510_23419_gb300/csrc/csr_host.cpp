@@ -6,8 +6,9 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdlib>
+#include <cstring>
+#include <future>
 #include <memory>
-#include <numeric>
 #include <string>
 #include <vector>
 
@@ -34,10 +35,13 @@ int greedy_colouring(int32_t N, int64_t E, const int32_t* eu, const int32_t* ev,
         adj[(size_t)fill[eu[e]]++] = ev[e];
         adj[(size_t)fill[ev[e]]++] = eu[e];
     }
-    std::vector<int32_t> order((size_t)N);
-    std::iota(order.begin(), order.end(), 0);
-    std::stable_sort(order.begin(), order.end(),
-                     [&](int32_t a, int32_t b) { return off[a + 1] - off[a] > off[b + 1] - off[b]; });
+    // by decreasing degree: bucket `first` of a degree starts after the larger ones'
+    int64_t most = 0;
+    for (int32_t i = 0; i < N; ++i) most = std::max(most, off[(size_t)i + 1] - off[i]);
+    std::vector<int32_t> order((size_t)N), first((size_t)most + 2, 0);
+    for (int32_t i = 0; i < N; ++i) first[(size_t)(most - (off[(size_t)i + 1] - off[i])) + 1]++;
+    for (int64_t d = 0; d <= most; ++d) first[(size_t)d + 1] += first[(size_t)d];
+    for (int32_t i = 0; i < N; ++i) order[(size_t)first[(size_t)(most - (off[(size_t)i + 1] - off[i]))]++] = i;
     std::fill(colour, colour + N, -1);
     std::vector<int64_t> seen;  // seen[c] == i: colour c is taken by a neighbour of i
     int k = 0;
@@ -55,6 +59,88 @@ int greedy_colouring(int32_t N, int64_t E, const int32_t* eu, const int32_t* ev,
         k = std::max(k, c + 1);
     }
     return k;
+}
+
+// Rows of the resident form (CsrResDevice) of a +-1 instance without fields.
+struct ResRows {
+    int npad = 0;  // 0: the instance has none
+    int regular = 1, rounds = 0, slot_rounds = 0, slot_words = 0;
+    std::vector<int32_t> pos, cls;
+    std::vector<uint16_t> nbr;
+    std::vector<uint32_t> sign, low, deg;
+};
+
+ResRows resident_rows(int32_t N, int k, int maxdeg, const std::vector<int32_t>& cls_off, const std::vector<int32_t>& rowptr,
+                      const std::vector<int32_t>& col, const std::vector<int8_t>& J8)
+{
+    ResRows r;
+    if (N > kCsrResSpins) return r;
+    r.pos.resize((size_t)N);
+    r.cls.assign((size_t)4 * k, 0);
+    std::vector<uint8_t> below((size_t)N);  // neighbours in lower classes
+    int npad = 0, slots = 0;
+    for (int c = 0; c < k; ++c) {
+        const int n0 = cls_off[(size_t)c], ncls = cls_off[(size_t)c + 1] - n0;
+        int32_t* cls = &r.cls[(size_t)4 * c];
+        cls[0] = npad / 4;
+        cls[1] = (ncls + 3) / 4;
+        cls[2] = ncls;
+        for (int q = 0; q < ncls; ++q) r.pos[(size_t)n0 + q] = npad + q;
+        npad += cls[1] * 4;
+        int lo = 0, hi = 0;  // widest lower and upper part of a row of the class, in even slot counts
+        for (int p = n0; p < n0 + ncls; ++p) {
+            const int32_t a0 = rowptr[(size_t)p], a1 = rowptr[(size_t)p + 1];
+            int under = 0;
+            for (int32_t a = a0; a < a1; ++a) under += col[(size_t)a] < n0;
+            below[(size_t)p] = (uint8_t)under;
+            lo = std::max(lo, under);
+            hi = std::max(hi, a1 - a0 - under);
+            if (a1 - a0 != maxdeg) r.regular = 0;
+        }
+        lo = (lo + 1) / 2 * 2;
+        hi = (hi + 1) / 2 * 2;
+        cls[3] = lo | ((lo + hi) << 16);
+        slots = std::max(slots, lo + hi);
+    }
+    if (npad > kCsrResSpins) return r;
+    int held = 0;  // words in a thread's energy count
+    for (int c = 0; c < k; ++c) {
+        int32_t* cls = &r.cls[(size_t)4 * c];
+        auto most = [](const int32_t* x) { return (x[1] + kCsrResThreads - 1) / kCsrResThreads; };
+        r.rounds += most(cls);
+        r.slot_rounds += most(cls) * (cls[3] >> 16);
+        r.slot_words += cls[1] * (cls[3] >> 16);
+        held += most(cls);
+        if (c + 1 < k && held + most(cls + 4) <= kCsrResWords) continue;
+        cls[3] |= kCsrResFlush;
+        held = 0;
+    }
+    const size_t words = (size_t)npad / 4;
+    r.nbr.assign((size_t)slots * npad, (uint16_t)npad);
+    r.sign.assign((size_t)slots * words, 0);
+    r.low.assign(words * 4, 0);
+    r.deg.assign(words, 0);
+    for (int c = 0; c < k; ++c) {
+        const int n0 = cls_off[(size_t)c], n1 = cls_off[(size_t)c + 1], lo = r.cls[(size_t)4 * c + 3] & 0xFF;
+        for (int p = n0; p < n1; ++p) {
+            const size_t at = (size_t)r.pos[(size_t)p], w = at / 4;
+            const int sh = 8 * (int)(at & 3);
+            const int32_t a0 = rowptr[(size_t)p], a1 = rowptr[(size_t)p + 1];
+            size_t u = at, v = at + (size_t)lo * npad;  // next lower and upper slot
+            for (int32_t a = a0; a < a1; ++a) {
+                const int q = col[(size_t)a];
+                size_t& slot = q < n0 ? u : v;
+                r.nbr[slot] = (uint16_t)r.pos[(size_t)q];
+                if (J8[(size_t)a] < 0) r.sign[slot / 4] |= 0xFFu << sh;
+                slot += (size_t)npad;
+            }
+            for (int b = 0, n = below[(size_t)p]; n; ++b, n >>= 1)
+                if (n & 1) r.low[4 * w + b] |= 0xFFu << sh;
+            r.deg[w] |= (uint32_t)(4 * (maxdeg - (a1 - a0))) << sh;
+        }
+    }
+    r.npad = npad;
+    return r;
 }
 
 }  // namespace
@@ -120,32 +206,38 @@ pb_status csr_build(pb_instance* I, int32_t N, int64_t E, const int32_t* eu, con
             else Jf[(size_t)a] = static_cast<const float*>(J)[e];
         }
     }
-    // +-1 rows: J = +1 half-edges first (stable), so the field walk needs no coupling
-    std::vector<int32_t> rowneg(pm1 ? (size_t)N : 0);
-    if (pm1) {
-        std::vector<int32_t> tc;
-        for (int32_t p = 0; p < N; ++p) {
-            const int32_t a0 = rowptr[p], a1 = rowptr[(size_t)p + 1];
-            tc.clear();
-            int32_t w = a0;
-            for (int32_t a = a0; a < a1; ++a) {
-                if (J8[(size_t)a] > 0) col[(size_t)w++] = col[(size_t)a];
-                else tc.push_back(col[(size_t)a]);
-            }
-            rowneg[(size_t)p] = w;
-            for (int32_t v : tc) col[(size_t)w++] = v;
-            for (int32_t a = a0; a < a1; ++a) J8[(size_t)a] = a < rowneg[(size_t)p] ? 1 : -1;
-        }
-    }
     int maxdeg = 0;
     for (int32_t p = 0; p < N; ++p) maxdeg = std::max(maxdeg, rowptr[(size_t)p + 1] - rowptr[p]);
+    // Resident rows, beside the other rows and their uploads (made after them, a quarter of a large instance's
+    // creation).  Small ones are made when they are asked for, as a thread costs more.
+    std::future<ResRows> res_rows;
+    if (pm1 && !h && maxdeg >= 1 && maxdeg <= kCsrResDegree)
+        res_rows = std::async(E >= 8192 ? std::launch::async | std::launch::deferred : std::launch::deferred, [&]() {
+            return resident_rows(N, k, maxdeg, cls_off, rowptr, col, J8);
+        });
+    // +-1 rows: J = +1 half-edges first (stable), so the field walk needs no coupling.  (Into new arrays: the resident
+    // rows are being made from the old ones.)
+    std::vector<int32_t> rowneg(pm1 ? (size_t)N : 0), colp(pm1 ? (size_t)(2 * E) : 0);
+    std::vector<int8_t> Jp(pm1 ? (size_t)(2 * E) : 0);
+    for (int32_t p = 0; pm1 && p < N; ++p) {
+        const int32_t a0 = rowptr[p], a1 = rowptr[(size_t)p + 1];
+        int32_t at[2] = {a0, a0};  // next J = +1 and J = -1 half-edge
+        for (int32_t a = a0; a < a1; ++a) at[1] += J8[(size_t)a] > 0;
+        rowneg[(size_t)p] = at[1];
+        for (int32_t a = a0; a < a1; ++a) {
+            const int32_t w = at[J8[(size_t)a] < 0]++;
+            colp[(size_t)w] = col[(size_t)a];
+            Jp[(size_t)w] = J8[(size_t)a];
+        }
+    }
+    const std::vector<int32_t>& rows = pm1 ? colp : col;
     // +-1, degree <= kCsrEllSlots: padded rows (unused slots name the zero row N)
     const bool ell = pm1 && maxdeg <= kCsrEllSlots;
     std::vector<int32_t> ellv(ell ? (size_t)N * kCsrEllSlots : 0, N);
     std::vector<uint16_t> ellnd(ell ? (size_t)N : 0);
     for (int32_t p = 0; ell && p < N; ++p) {
         const int32_t a0 = rowptr[p], a1 = rowptr[(size_t)p + 1];
-        for (int32_t a = a0; a < a1; ++a) ellv[(size_t)p * kCsrEllSlots + (a - a0)] = col[(size_t)a];
+        for (int32_t a = a0; a < a1; ++a) ellv[(size_t)p * kCsrEllSlots + (a - a0)] = rows[(size_t)a];
         ellnd[(size_t)p] = (uint16_t)((rowneg[(size_t)p] - a0) | ((a1 - a0) << 8));
     }
     // per-label colour and field
@@ -174,99 +266,48 @@ pb_status csr_build(pb_instance* I, int32_t N, int64_t E, const int32_t* eu, con
     I->n_colours = k;
     I->csr_cls_off = cls_off;
     I->csr_orig = orig;
-    // resident rows
-    const bool res = pm1 && !h && maxdeg >= 1 && maxdeg <= kCsrResDegree;
-    std::vector<int32_t> rpos, rcls;
-    std::vector<uint16_t> rnbr;
-    std::vector<uint32_t> rsign, rdeg;
-    std::vector<uint32_t> rlow;
-    int npad = 0, rslots = 0, rrounds = 0, rslot_rounds = 0, rslot_words = 0;
-    if (res) {
-        rpos.resize((size_t)N);
-        rcls.assign((size_t)4 * k, 0);
-        for (int c = 0; c < k; ++c) {
-            const int n0 = cls_off[(size_t)c], ncls = cls_off[(size_t)c + 1] - n0;
-            rcls[(size_t)4 * c] = npad / 4;
-            rcls[(size_t)4 * c + 1] = (ncls + 3) / 4;
-            rcls[(size_t)4 * c + 2] = ncls;
-            for (int q = 0; q < ncls; ++q) rpos[(size_t)n0 + q] = npad + q;
-            npad += (ncls + 3) / 4 * 4;
-            int lo = 0, hi = 0;  // widest lower and upper part of a row of the class, in even slot counts
-            for (int p = n0; p < n0 + ncls; ++p) {
-                int below = 0;
-                for (int32_t a = rowptr[(size_t)p]; a < rowptr[(size_t)p + 1]; ++a) below += col[(size_t)a] < n0;
-                lo = std::max(lo, below);
-                hi = std::max(hi, rowptr[(size_t)p + 1] - rowptr[(size_t)p] - below);
-            }
-            lo = (lo + 1) / 2 * 2;
-            hi = (hi + 1) / 2 * 2;
-            rcls[(size_t)4 * c + 3] = lo | ((lo + hi) << 16);
-            rslots = std::max(rslots, lo + hi);
-        }
-        int held = 0;  // words in a thread's energy count
-        for (int c = 0; c < k; ++c) {
-            const int ro = (rcls[(size_t)4 * c + 1] + kCsrResThreads - 1) / kCsrResThreads;
-            rrounds += ro;
-            rslot_rounds += ro * (rcls[(size_t)4 * c + 3] >> 16);
-            rslot_words += rcls[(size_t)4 * c + 1] * (rcls[(size_t)4 * c + 3] >> 16);
-            auto most = [&](int cc) { return (rcls[(size_t)4 * cc + 1] + kCsrResThreads - 1) / kCsrResThreads; };
-            held += most(c);
-            if (c + 1 < k && held + most(c + 1) <= kCsrResWords) continue;
-            rcls[(size_t)4 * c + 3] |= kCsrResFlush;
-            held = 0;
-        }
-    }
-    const bool res_fits = res && npad <= kCsrResSpins;
-    if (res_fits) {
-        const size_t words = (size_t)npad / 4;
-        rnbr.assign((size_t)rslots * npad, (uint16_t)npad);
-        rsign.assign((size_t)rslots * words, 0);
-        rlow.assign(words * 4, 0);
-        rdeg.assign(words, 0);
-        for (int c = 0; c < k; ++c) {
-            const int n0 = cls_off[(size_t)c], n1 = cls_off[(size_t)c + 1], lo = rcls[(size_t)4 * c + 3] & 0xFF;
-            for (int p = n0; p < n1; ++p) {
-                const int at = rpos[(size_t)p], w = at / 4, j = at & 3;
-                int sl = 0, sh = lo;
-                for (int32_t a = rowptr[(size_t)p]; a < rowptr[(size_t)p + 1]; ++a) {
-                    const int q = col[(size_t)a];
-                    const int u = q < n0 ? sl++ : sh++;
-                    rnbr[((size_t)u * words + w) * 4 + j] = (uint16_t)rpos[(size_t)q];
-                    if (J8[(size_t)a] < 0) rsign[(size_t)u * words + w] |= 0xFFu << (8 * j);
-                }
-                for (int b = 0; b < 4; ++b)
-                    if ((sl >> b) & 1) rlow[4 * (size_t)w + b] |= 0xFFu << (8 * j);
-                rdeg[(size_t)w] |= (uint32_t)(4 * (maxdeg - (rowptr[(size_t)p + 1] - rowptr[(size_t)p]))) << (8 * j);
-            }
-        }
-    }
-    DevBuf* B = I->csr_bufs;  // 0 rowptr, 1 col, 2 J, 3 h, 4 cls_off, 5 orig, 6 colour, 7 rowneg, 8 pos
-    auto up = [&](DevBuf& b, const void* src, size_t bytes) -> pb_status {
-        PB_ALLOC(b, bytes);
-        if (bytes) PB_CUDA_TRY(cudaMemcpyAsync(b.p, src, bytes, cudaMemcpyHostToDevice, st));
-        return PB_OK;
+    // One device block, parts on 256-byte boundaries.  A small instance goes up in one copy (each cost 5 us).
+    struct Part {
+        const void* src;
+        size_t bytes, off;
     };
-    pb_status ps;
-    if ((ps = up(B[0], rowptr.data(), rowptr.size() * 4)) != PB_OK) return ps;
-    if ((ps = up(B[1], col.data(), col.size() * 4)) != PB_OK) return ps;
-    if ((ps = pm1 ? up(B[2], J8.data(), J8.size()) : up(B[2], Jf.data(), Jf.size() * 4)) != PB_OK) return ps;
-    if (h && (ps = pm1 ? up(B[3], h8l.data(), h8l.size()) : up(B[3], hfl.data(), hfl.size() * 4)) != PB_OK) return ps;
-    if ((ps = up(B[4], cls_off.data(), cls_off.size() * 4)) != PB_OK) return ps;
-    if ((ps = up(B[5], orig.data(), orig.size() * 4)) != PB_OK) return ps;
-    if ((ps = up(B[6], colour_l.data(), colour_l.size() * 4)) != PB_OK) return ps;
-    if (pm1 && (ps = up(B[7], rowneg.data(), rowneg.size() * 4)) != PB_OK) return ps;
-    if ((ps = up(B[8], pos.data(), pos.size() * 4)) != PB_OK) return ps;
-    if (ell && (ps = up(B[9], ellv.data(), ellv.size() * 4)) != PB_OK) return ps;
-    if (ell && (ps = up(B[10], ellnd.data(), ellnd.size() * 2)) != PB_OK) return ps;
-    if (res_fits) {
-        if ((ps = up(B[11], rnbr.data(), rnbr.size() * 2)) != PB_OK) return ps;
-        if ((ps = up(B[12], rsign.data(), rsign.size() * 4)) != PB_OK) return ps;
-        if ((ps = up(B[13], rlow.data(), rlow.size() * 4)) != PB_OK) return ps;
-        if ((ps = up(B[14], rdeg.data(), rdeg.size() * 4)) != PB_OK) return ps;
-        if ((ps = up(B[15], rcls.data(), rcls.size() * 4)) != PB_OK) return ps;
-        if ((ps = up(B[16], rpos.data(), rpos.size() * 4)) != PB_OK) return ps;
+    std::vector<Part> parts;
+    size_t total = 0;
+    auto add = [&](const void* src, size_t bytes) {
+        parts.push_back({src, bytes, total});
+        total += (bytes + 255) / 256 * 256;
+        return parts.back().off;
+    };
+    enum { kRowptr, kCol, kJ, kH, kClsOff, kOrig, kColour, kRowneg, kPos, kEll, kEllNd, kNbr, kSign, kLow, kDeg, kCls, kResPos };
+    add(rowptr.data(), rowptr.size() * 4);
+    add(rows.data(), rows.size() * 4);
+    pm1 ? add(Jp.data(), Jp.size()) : add(Jf.data(), Jf.size() * 4);
+    pm1 ? add(h8l.data(), h8l.size()) : add(hfl.data(), hfl.size() * 4);
+    add(cls_off.data(), cls_off.size() * 4);
+    add(orig.data(), orig.size() * 4);
+    add(colour_l.data(), colour_l.size() * 4);
+    add(rowneg.data(), rowneg.size() * 4);
+    add(pos.data(), pos.size() * 4);
+    add(ellv.data(), ellv.size() * 4);
+    add(ellnd.data(), ellnd.size() * 2);
+    const ResRows r = res_rows.valid() ? res_rows.get() : ResRows{};
+    add(r.nbr.data(), r.nbr.size() * 2);
+    add(r.sign.data(), r.sign.size() * 4);
+    add(r.low.data(), r.low.size() * 4);
+    add(r.deg.data(), r.deg.size() * 4);
+    add(r.cls.data(), r.npad ? r.cls.size() * 4 : 0);
+    add(r.pos.data(), r.npad ? r.pos.size() * 4 : 0);
+    PB_ALLOC(I->csr_buf, total);
+    char* const base = I->csr_buf.as<char>();
+    std::vector<char> stage(total <= ((size_t)512 << 10) ? total : 0);
+    for (const Part& q : parts) {
+        if (q.bytes == 0) continue;
+        if (!stage.empty()) std::memcpy(stage.data() + q.off, q.src, q.bytes);
+        else PB_CUDA_TRY(cudaMemcpyAsync(base + q.off, q.src, q.bytes, cudaMemcpyHostToDevice, st));
     }
+    if (!stage.empty()) PB_CUDA_TRY(cudaMemcpyAsync(base, stage.data(), total, cudaMemcpyHostToDevice, st));
     PB_CUDA_TRY(cudaStreamSynchronize(st));
+    auto at = [&](int k) { return static_cast<void*>(base + parts[(size_t)k].off); };
     CsrDevice& g = I->csr;
     g = CsrDevice{};
     g.N = N;
@@ -275,34 +316,32 @@ pb_status csr_build(pb_instance* I, int32_t N, int64_t E, const int32_t* eu, con
     g.maxdeg = maxdeg;
     g.has_h = I->has_h;
     g.hmax = hmax;
-    g.rowptr = B[0].as<int32_t>();
-    g.col = B[1].as<int32_t>();
-    g.rowneg = pm1 ? B[7].as<int32_t>() : nullptr;
-    g.J8 = pm1 ? B[2].as<int8_t>() : nullptr;
-    g.Jf = pm1 ? nullptr : B[2].as<float>();
-    g.h8 = (h && pm1) ? B[3].as<int8_t>() : nullptr;
-    g.hf = (h && !pm1) ? B[3].as<float>() : nullptr;
-    g.cls_off = B[4].as<int32_t>();
-    g.orig = B[5].as<int32_t>();
-    g.pos = B[8].as<int32_t>();
-    g.colour = B[6].as<int32_t>();
-    g.ell = ell ? B[9].as<int4>() : nullptr;
-    g.ell_nd = ell ? B[10].as<uint16_t>() : nullptr;
-    if (res_fits) {
-        g.res.npad = npad;
-        g.res.regular = 1;
-        for (int32_t p = 0; p < N; ++p)
-            if (rowptr[(size_t)p + 1] - rowptr[p] != maxdeg) g.res.regular = 0;
+    g.rowptr = static_cast<int32_t*>(at(kRowptr));
+    g.col = static_cast<int32_t*>(at(kCol));
+    g.rowneg = pm1 ? static_cast<int32_t*>(at(kRowneg)) : nullptr;
+    g.J8 = pm1 ? static_cast<int8_t*>(at(kJ)) : nullptr;
+    g.Jf = pm1 ? nullptr : static_cast<float*>(at(kJ));
+    g.h8 = (h && pm1) ? static_cast<int8_t*>(at(kH)) : nullptr;
+    g.hf = (h && !pm1) ? static_cast<float*>(at(kH)) : nullptr;
+    g.cls_off = static_cast<int32_t*>(at(kClsOff));
+    g.orig = static_cast<int32_t*>(at(kOrig));
+    g.pos = static_cast<int32_t*>(at(kPos));
+    g.colour = static_cast<int32_t*>(at(kColour));
+    g.ell = ell ? static_cast<int4*>(at(kEll)) : nullptr;
+    g.ell_nd = ell ? static_cast<uint16_t*>(at(kEllNd)) : nullptr;
+    if (r.npad) {
+        g.res.npad = r.npad;
+        g.res.regular = r.regular;
         g.res.edges = (int32_t)E;
-        g.res.nbr = B[11].as<uint2>();
-        g.res.sign = B[12].as<uint32_t>();
-        g.res.lowdeg = B[13].as<uint4>();
-        g.res.degoff = B[14].as<uint32_t>();
-        g.res.cls = B[15].as<int32_t>();
-        g.res.pos = B[16].as<int32_t>();
-        g.res.rounds = rrounds;
-        g.res.slot_rounds = rslot_rounds;
-        g.res.slot_words = rslot_words;
+        g.res.nbr = static_cast<uint2*>(at(kNbr));
+        g.res.sign = static_cast<uint32_t*>(at(kSign));
+        g.res.lowdeg = static_cast<uint4*>(at(kLow));
+        g.res.degoff = static_cast<uint32_t*>(at(kDeg));
+        g.res.cls = static_cast<int32_t*>(at(kCls));
+        g.res.pos = static_cast<int32_t*>(at(kResPos));
+        g.res.rounds = r.rounds;
+        g.res.slot_rounds = r.slot_rounds;
+        g.res.slot_words = r.slot_words;
     }
     return PB_OK;
 }
