@@ -463,7 +463,7 @@ pb_status ea_batch_setup(std::vector<pb_run*>& runs, cudaStream_t st, std::share
     bool f32_l24 = false, f32_l32 = false;
     for (const pb_run* r : runs) {
         if (r->job.inst.jtype != PB_J_F32) continue;
-        f32_l24 |= r->job.inst.jtype == PB_J_F32 && r->job.inst.L * r->job.inst.L * r->job.WT == 576;
+        f32_l24 |= r->job.inst.L * r->job.inst.L * r->job.WT == 576;
         f32_l32 |= ea_tile_path(r->job) == kEaPathFast32;
     }
     bool split = true;
