@@ -816,7 +816,7 @@ CASES = {
     "bq-n1024-R1024-pm1-tensor": ("bq", 1024, "pm1", 1024, 4, "tensor"),
     "bq-n4096-R4096-pm1-tensor-s200": ("bq", 4096, "pm1", 4096, 200, "tensor"),
     "bq-n4096-R4096-gauss-tensor-s100": ("bq", 4096, "gauss", 4096, 100, "tensor"),
-    "csr-cube25-R1024-pm1": ("csr", 25, "pm1", 1024, 50, "plain"),
+    "csr-cube25-R1024-pm1": ("csr", 25, "pm1", 1024, 50, "auto"),  # the resident form
 }
 
 
@@ -831,8 +831,8 @@ def run_case(name, sweeps=None):
     if sweeps:
         S = sweeps
     dist = {"pm1": pb.PB_DIST_PM1, "gauss": pb.PB_DIST_GAUSS, "unif": pb.PB_DIST_UNIF}[law]
-    forms = {"resident": pb.PB_FORM_RESIDENT, "plain": pb.PB_FORM_PLAIN, "cudacore": pb.PB_FORM_CUDACORE,
-             "tensor": pb.PB_FORM_TENSOR}
+    forms = {"auto": pb.PB_FORM_AUTO, "resident": pb.PB_FORM_RESIDENT, "plain": pb.PB_FORM_PLAIN,
+             "cudacore": pb.PB_FORM_CUDACORE, "tensor": pb.PB_FORM_TENSOR}
     if topo == "ea":
         J = pb.pb_generate_ea(size, dist, 3)
         inst = pb.pb_create_instance(pb.PB_TOPO_EA3D, J, None, L=size)
