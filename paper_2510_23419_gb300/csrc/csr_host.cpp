@@ -1,6 +1,6 @@
 // csr_host.cpp -- general sparse instances (arXiv 2510.23419, Eq. 1 on an
 // arbitrary edge set; update groups of Sec. 1.2.2 from a proper colouring):
-// instance build, greedy colouring, runs of the plain per-class form.
+// instance build, greedy colouring, runs of the resident and of the plain per-class form.
 #include <cuda_runtime.h>
 
 #include <algorithm>

@@ -13,7 +13,7 @@
 // threshold lookup and a compare.  The per-class launches that this replaces kept a
 // byte per spin and replica in global memory and took 68 instructions per update
 // and 5 launches per sweep on the L = 25 cube (4 colours): us per sweep, before -> after: 1024
-// replicas 68.8 -> 26.5, 64 replicas 34.9 -> 19.5; L = 11, 256 replicas 27.9 -> 5.1.  What bounds it now: the
+// replicas 70.3 -> 28.4, 64 replicas 34.7 -> 19.7; L = 11, 256 replicas 28.9 -> 5.7.  What bounds it now: the
 // part-filled rounds of a class (its words over 512 threads) and L2 latency of the rows; more
 // threads did not help (768: 29.0, 1024: 29.4 us against 27.8 at 512 then).
 //

@@ -41,7 +41,7 @@ int64_t footprint_bytes(const pb_instance* I, const pb_schedule* sc, int R, cons
     const int64_t nlev = std::max<int64_t>(1, (int64_t)betas.size());
     int form = 0, wt = 0;
     choose_form(I, R, opts ? opts->form : PB_FORM_AUTO, form, wt);
-    if (form == kFormResidentWide) form = PB_FORM_TENSOR;  // admitted by the footprint of the form it replaces, the larger one
+    if (form == kFormResidentWide) form = PB_FORM_TENSOR;  // admitted by the footprint of the tensor form, the larger one
     const int64_t N = I->N;
     const int64_t out = 2 * (int64_t)R * N + 2 * (int64_t)R * 8;  // readout states and energies
     if (I->topo == PB_TOPO_EA3D) {
